@@ -107,15 +107,10 @@ struct KTime {
     int kernels;   // kernel launches per step in this stage
 };
 // the step graph: rebuild = one-pass scan, scatter, gather (the keys and histogram come from
-// the previous step's update); the update also computes the next keys, and is two kernels
-// (viscous sum, update) where SPH_SPLIT_INTEGRATE_2D/3D says so
+// the previous step's update); interact = search, pressure pass; integrate = prediction, viscous
+// sum, update (which also computes the next keys)
 constexpr int NSTAGE = 4;
-const KTime kStages[NSTAGE] = {{"rebuild", 3}, {"interact", 1}, {"control", 1}, {"integrate", 1}};
-int stage_kernels(int k, int D) {
-    if (k == 3) return (D == 2 ? SPH_SPLIT_INTEGRATE_2D : SPH_SPLIT_INTEGRATE_3D) ? 2 : 1;
-    return kStages[k].kernels;
-}
-
+const KTime kStages[NSTAGE] = {{"rebuild", 3}, {"interact", 2}, {"control", 1}, {"integrate", 3}};
 // host copy of one instance
 struct Inst {
     Grid grid;            // base[] and occ_base are global (set by relayout)
@@ -194,10 +189,9 @@ template <> State<double>& st<double>(sph_batch* b) { return b->sd; }
 // cell keys of a batch (int32 keys and cell starts; the one-pass scan has no other bound)
 constexpr long long MAX_KEYS = 1ll << 30;
 
-int lpp_of(int D) { return D == 2 ? Lpp<2>::v : Lpp<3>::v; }
+int list_entries_of(int D) { return D == 2 ? list_entries<2>() : list_entries<3>(); }
 // cells per support when the parameters leave it to the library (measured per dimension)
 int default_cps(int D) { return D == 2 ? SPH_DEFAULT_CPS_2D : SPH_DEFAULT_CPS_3D; }
-int vcap_of(int D) { return D == 2 ? Vcap<2>::v : Vcap<3>::v; }
 
 // Validates one instance's descriptors and fills its host copy (grid bases instance-relative).
 sph_status make_instance(const sph_domain_desc* dd, const sph_sizing_desc* sz, const sph_params* pp,
@@ -426,9 +420,7 @@ void ctrl_inf_bits(int prec, Ctrl* c) {
 // carve the per-slot arrays out of one allocation (256-byte aligned pieces)
 template <typename T> size_t slot_layout(sph_batch* b, char* base, bool assign) {
     const size_t cap = (size_t)std::max(b->slot_cap, 1);
-    const size_t nlanes = cap * (size_t)lpp_of(b->D);
-    const size_t nblk = (size_t)div_up((long long)nlanes, BLOCK);
-    const size_t vcap = (size_t)vcap_of(b->D);
+    const size_t nlist = cap * (size_t)list_entries_of(b->D);   // cap: whole chunks
     size_t off = 0;
     auto take = [&](size_t bytes) -> char* {
         off = (off + 255) & ~(size_t)255;
@@ -438,7 +430,7 @@ template <typename T> size_t slot_layout(sph_batch* b, char* base, bool assign) 
     };
     State<T> s;
     std::memset(&s, 0, sizeof s);
-    for (int a = 0; a < 3; ++a) {
+    for (int a = 0; a < b->D; ++a) {
         s.C[a] = (int*)take(cap * 4);
         s.O[a] = (T*)take(cap * sizeof(T));
         s.V[a] = (T*)take(cap * sizeof(T));
@@ -450,23 +442,25 @@ template <typename T> size_t slot_layout(sph_batch* b, char* base, bool assign) 
     s.G = (unsigned*)take(cap * 4);
     s.ID = (int*)take(cap * 4);
     s.K = (int*)take(cap * 4);
-    s.Ms = (unsigned*)take(cap * 4);
+    s.Ms = (unsigned*)take(cap * (b->D == 2 ? sizeof(Meta<2>) : sizeof(Meta<3>)));
     s.IDs = (int*)take(cap * 4);
     s.Ks = (int*)take(cap * 4);
     s.P = (Vec4<T>*)take(cap * sizeof(Vec4<T>));
+    s.F = (float4*)take(cap * sizeof(float4));
     s.A = (Vec4<T>*)take(cap * sizeof(Vec4<T>));
     s.perm = (int*)take(cap * 4);
     s.sperm = (int*)take(cap * 4);
-    s.partials = (double*)take(nblk * MAXF * sizeof(double));
     s.partials2 = (double*)take((cap / CHUNK + 1) * MAXF * sizeof(double));
     s.pticket = (int*)take((cap / CHUNK + 1) * sizeof(int));
-    s.vj = (int*)take(nlanes * vcap * 4);
-    s.vr = (T*)take(nlanes * vcap * sizeof(T));
-    s.vcnt = (int*)take(nlanes * 4);
+    s.vj = (int*)take(nlist * 4);
+    s.vr = (T*)take(nlist * sizeof(T));
+    s.vcnt = (int*)take(cap * 4);
+    s.xid = (unsigned long long*)take(cap * 8);
+    s.xcnt = (int*)take((cap / CHUNK + 1) * sizeof(int));
+    s.xbase = cap * (size_t)(b->D == 2 ? ListShape<2>::ROW : ListShape<3>::ROW);
     if (assign) {
         s.n = b->nslots;
         s.NI = b->NI;
-        s.nblk = div_up((long long)b->nslots * lpp_of(b->D), BLOCK);
         s.inst_off = b->d_inst_off;
         s.inst_n = b->d_inst_n;
         s.chunk_inst = b->d_chunk_inst;
@@ -505,7 +499,6 @@ template <typename T, int D> void repack(sph_batch* b) { launch_repack<T, D>(st<
 template <typename T> void set_slots(sph_batch* b) {
     State<T>& s = st<T>(b);
     s.n = b->nslots;
-    s.nblk = div_up((long long)b->nslots * lpp_of(b->D), BLOCK);
 }
 
 // Lays the batch out again after instance `changed` gets `new_n` particles (changed < 0: no
@@ -661,7 +654,7 @@ sph_status batch_init(sph_batch* b, void* stream) {
         I.n = 0;
         cap += std::max<int64_t>(CHUNK, (I.cap + CHUNK - 1) / CHUNK * CHUNK);
     }
-    if (cap * 12 >= ((long long)1 << 31))   // lane-indexed arrays hold slots * LPP * VCAP entries
+    if (cap * 12 >= ((long long)1 << 31))   // lane indices of the pair passes are 32-bit
         return fail(SPH_E_INVALID, "batch: %lld particle slots in total is too many", cap);
     b->slot_cap = (int)cap;
     b->nslots = 0;
@@ -751,7 +744,8 @@ template <typename T, int D> void enqueue_step(sph_batch* b, bool timed) {
             if (timed && first) cudaEventRecordWithFlags(b->ev[0], stream, cudaEventRecordExternal);
             enqueue_rebuild<T, D>(b, s, stream);
             if (timed && first) cudaEventRecordWithFlags(b->ev[1], stream, cudaEventRecordExternal);
-            launch_interact<T, D>(s, one_of(b), nullptr, nullptr, stream, !timed, cls);
+            launch_search<T, D>(s, one_of(b), stream, !timed, cls);
+            launch_interact<T, D>(s, one_of(b), nullptr, nullptr, stream, true, cls);
             if (timed && first) cudaEventRecordWithFlags(b->ev[2], stream, cudaEventRecordExternal);
             launch_control<T, D>(s, one_of(b), stream, !timed, cls);
             if (timed && first) cudaEventRecordWithFlags(b->ev[3], stream, cudaEventRecordExternal);
@@ -765,7 +759,8 @@ template <typename T, int D> void enqueue_step(sph_batch* b, bool timed) {
     if (timed) cudaEventRecordWithFlags(b->ev[1], stream, cudaEventRecordExternal);
     // kernel-to-kernel edges start the successor early (programmatic dependent launch); an
     // event between two kernels makes the edge an ordinary one
-    launch_interact<T, D>(s, one_of(b), nullptr, nullptr, stream, !timed);
+    launch_search<T, D>(s, one_of(b), stream, !timed);
+    launch_interact<T, D>(s, one_of(b), nullptr, nullptr, stream, true);
     if (timed) cudaEventRecordWithFlags(b->ev[2], stream, cudaEventRecordExternal);
     launch_control<T, D>(s, one_of(b), stream, !timed);
     if (timed) cudaEventRecordWithFlags(b->ev[3], stream, cudaEventRecordExternal);
@@ -1056,6 +1051,7 @@ sph_status dbg_neighbors_impl(sph_batch* b, int32_t mode, int64_t* counts_out, i
     long long* d_off = nullptr;
     int* d_lists = nullptr;
     CK(cudaMalloc(&d_counts, 4 * (size_t)std::max(ns, 1)));
+    launch_search<T, D>(s, one_of(b), b->stream, false, -1);
     launch_neighbors<T, D>(s, mode, d_counts, nullptr, nullptr, b->stream);
     std::vector<int> cnt(ns), ids(ns);
     CK(cudaMemcpyAsync(cnt.data(), d_counts, 4 * (size_t)ns, cudaMemcpyDeviceToHost, b->stream));
@@ -1107,6 +1103,7 @@ sph_status dbg_interact_impl(sph_batch* b, double* a_p, double* sigma, double* g
     T *d_sig = nullptr, *d_gam = nullptr;
     CK(cudaMalloc(&d_sig, sizeof(T) * (size_t)std::max(ns, 1)));
     CK(cudaMalloc(&d_gam, sizeof(T) * (size_t)std::max(ns, 1)));
+    launch_search<T, D>(s, one_of(b), b->stream);
     launch_interact<T, D>(s, one_of(b), d_sig, d_gam, b->stream);
     CK(cudaGetLastError());
     std::vector<Vec4<T>> A(ns);
@@ -1169,6 +1166,7 @@ sph_status dbg_update_impl(sph_batch* b, const double* dt, const int32_t* reset,
     State<T> s;
     sph_status r = dbg_prepare<T, D>(b, s, &c);
     if (r != SPH_OK) return r;
+    launch_search<T, D>(s, one_of(b), b->stream);
     launch_interact<T, D>(s, one_of(b), nullptr, nullptr, b->stream);
     // scratch output arrays
     Out<T> o;
@@ -1209,7 +1207,8 @@ template <typename T, int D> sph_status pair_counts_impl(sph_batch* b, int64_t* 
     unsigned long long* d = nullptr;
     CK(cudaMalloc(&d, 16));
     CK(cudaMemsetAsync(d, 0, 16, b->stream));
-    launch_pair_counts<T, D>(s, d, b->stream);
+    launch_search<T, D>(s, one_of(b), b->stream, false, -1, d);
+    launch_pair_counts<T, D>(s, d + 1, b->stream);
     unsigned long long h[2];
     CK(cudaMemcpyAsync(h, d, 16, cudaMemcpyDeviceToHost, b->stream));
     CK(cudaStreamSynchronize(b->stream));
@@ -1565,7 +1564,7 @@ sph_status kernel_times_impl(sph_batch* b, sph_kernel_time* out, int32_t cap, in
     for (; k < NSTAGE && k < cap; ++k) {
         std::memset(out[k].name, 0, sizeof out[k].name);
         std::snprintf(out[k].name, sizeof out[k].name, "%s", kStages[k].name);
-        out[k].launches = b->stage_steps * stage_kernels(k, b->D);
+        out[k].launches = b->stage_steps * kStages[k].kernels;
         out[k].total_ms = b->stage_ms[k];
     }
     if (n_out) *n_out = k;

@@ -1,7 +1,7 @@
 // integrate.cu -- per-step controller (Sec. 3.4, Eq. 24) and the viscous pass + update +
 // projection of one relaxation step (Algorithm 1: mid-point velocity, viscous force, map,
 // predicted velocity, position, map).
-#include "sph_internal.cuh"
+#include "walk.cuh"
 
 namespace sph {
 
@@ -467,98 +467,35 @@ template <typename T> __device__ __forceinline__ T domain_phi_t(const Domain& do
     return phi;
 }
 
-// Viscous pass + update, one thread per sorted particle, writing the new state in sorted order:
+// Viscous pass and update, writing the new state in sorted order:
 //   v'_i = 0 (nullified) or f v_i;  v~_i = v'_i + dt (a_p,i - eps v'_i)                       (Eq. 23)
 //   a_v,i = Pi_i sum_{j in g, j != i} [2 eta_i eta_j/(eta_i+eta_j)] (rho_i^-2 + rho_j^-2)
 //                 W_d'(r_ij, h_ij) (v~_i - v~_j) / r_ij,  eta = rho nu, nu = visc r_c |v~|    (Eq. 7, Eq. 8)
 //   v+ = v~ + dt a_v;  x+ = x + dt v+  (FP64);  curves/surfaces: x+ onto the feature in FP64,
 //   v+ <- Pi(x+) v+;  volume: phi(x+) < 0 -> back to phi = 0.01 h along grad phi (FP64),
 //   v+ = 0, escape counted;  h+ = h_t(x+).
-// The neighbour sum runs over the same-group pairs the pressure pass handed over (its LPI
-// list columns per particle, LPI/LPP of them per lane of this pass), or, where a column
-// overflowed, over the walk of the pressure pass (same pairs, same predicate) with LPP lanes;
-// the lead lane does the update.  As in the pressure pass, a block lies in one instance.
-// Padding slots are copied through unchanged.
-// MODE 0 runs both parts; MODE 1 only the viscous sum, leaving the projected a_v of each moving
-// particle in o.V (the stored velocities, which nothing reads during a step once the rebuild
-// has gathered them); MODE 2 (one lane per particle) only the update, taking a_v from o.V.
-template <typename T, int D, int MODE> constexpr int integrate_minb() {
-    if (sizeof(T) != 4) return 4;
-    if (MODE == 1) return D == 2 ? SPH_VISC_MINB_2D : SPH_VISC_MINB_3D;
-    if (MODE == 2) return SPH_UPDATE_MINB;
-    return D == 2 ? SPH_INTEGRATE_MINB_2D : SPH_INTEGRATE_MINB_3D;
+// Three kernels: k_predict turns the pressure pass's (a_p, V~) records into (v~, eta), so that a
+// pair of the viscous sum loads one record of its neighbour and computes no root or power; k_visc
+// sums over the lists with the kernel factors the pressure pass wrote, LPP lanes per particle
+// (particles whose list overflowed are searched again), leaving the projected a_v of each moving
+// particle in o.V (the stored velocities, which nothing reads during a step once the rebuild has
+// gathered them); k_update moves the particles, taking a_v from o.V.  The viscous sum is bound by the
+// latency of its chains list -> record (DRAM 30 %); with the neighbour's root, powers and quotient
+// computed per pair, from two records, sum and update of the 1.2M cube took 0.53 ms, now 0.36.  Small batches are bound by the
+// chain of launches and take one kernel for all (FUSED): every pair predicts its neighbour itself.
+
+// whether particle k (group gi, dimension di) moves in this pass: a converged instance (or, with
+// group_convergence, group) stays put
+__device__ __forceinline__ bool moves(const Params& p, const Ctrl* cu, int gi, int di, int cls, int D) {
+    if (di == 0 || cu->phase == PH_DONE || !in_pass(p, cls, di, D)) return false;
+    return !(p.group_conv && cu->gphase[gi] == PH_DONE);
 }
-template <typename T, int D, bool ONE, int MODE>
-__global__ void __launch_bounds__(BLOCK, (integrate_minb<T, D, MODE>()))
-    k_integrate(State<T> s, One one, const Ctrl* use, Out<T> o, int cls) {
-    dep_launch();
-    dep_wait();
-    constexpr int LPP = MODE == 2 ? 1 : ILpp<D>::v, LPI = Lpp<D>::v, NCOL = LPI / LPP;
-    __shared__ int2 sbuf[BUF_CAP * BLOCK];
-    __shared__ Grid gsh;
-    __shared__ Params psh;
-    const int inst = ONE ? 0 : __ldg(s.chunk_inst + (blockIdx.x * (BLOCK / LPP)) / CHUNK);
-    const Ctrl* const cu = use + inst;
-    Ctrl* const ctrl = s.ctrls + inst;
-    const Domain& dom = s.doms[inst];
-    if (!ONE) {
-        block_copy(&gsh, s.grids + inst);
-        block_copy(&psh, s.params + inst);
-        __syncthreads();
-    }
-    const Grid& g = ONE ? one.g : gsh;
-    const Params& p = ONE ? one.p : psh;
-    if (MODE != 1 && o.K) reset_scan_state(s);   // this kernel produces the next scan's histogram
-    const int k = (blockIdx.x * blockDim.x + threadIdx.x) / LPP;
-    const bool lead = (threadIdx.x % LPP) == 0;
-    if (MODE != 1 && k < s.n && !live(s, inst, k)) {   // padding: keep the slot as it is
-        if (lead) {
-            const Vec4<T> vh = s.VH[k];
-            const T vv[3] = {vh.x, vh.y, vh.z};
-            for (int a = 0; a < D; ++a) {
-                o.C[a][k] = s.Cs[a][k];
-                o.O[a][k] = s.Os[a][k];
-                o.V[a][k] = vv[a];
-                if (o.av[a]) o.av[a][k] = T(0);
-            }
-            o.H[k] = vh.w;
-            o.G[k] = 0u;
-            o.ID[k] = s.IDs[k];
-            if (o.K) {   // the next rebuild's key: the instance's dummy cell
-                o.K[k] = g.base[MAXL];
-                atomicAdd(o.count + g.base[MAXL], 1);
-            }
-        }
-    }
-    const bool inrange = k < s.n && live(s, inst, k);
-    T offi[3] = {T(0), T(0), T(0)}, hi = T(1);
-    unsigned mi = 0;
-    int c[3] = {0, 0, 0};            // stored position: finest cell + offset
-    T o3[3] = {T(0), T(0), T(0)};
-    T v[3] = {T(0), T(0), T(0)};
-    if (inrange) {
-        Rec<T, D>::load(s.P, s.Ms, k, offi, hi, mi);
-        const Vec4<T> vh = s.VH[k];
-        const T vv[3] = {vh.x, vh.y, vh.z};
-        for (int a = 0; a < D; ++a) {
-            c[a] = s.Cs[a][k];
-            o3[a] = s.Os[a][k];
-            v[a] = vv[a];
-        }
-    }
-    const int gi = inrange ? meta_group(mi) : -1, di = inrange ? meta_dim(mi) : 0;
-    // a converged instance (or, with group_convergence, group) stays put; the instance's
-    // scalars need no load that waits for the particle's group
-    bool done = cu->phase == PH_DONE;
-    if (p.group_conv && !done && inrange && di > 0) done = cu->gphase[gi] == PH_DONE;
-    const bool moving = inrange && di > 0 && !done && in_pass(p, cls, di, D);
-    T av[3] = {T(0), T(0), T(0)};
-    T hnew = hi;
-    T dt = T(0), f = T(1), eps = T(0);
-    bool rs = true;
-    T vt[3] = {T(0), T(0), T(0)};
-    T tg[3] = {T(0), T(0), T(0)};
-    if (moving) {
+
+// the step parameters of a group
+template <typename T> struct StepOf {
+    T dt, f, eps;
+    bool rs;
+    __device__ __forceinline__ StepOf(const Params& p, const Ctrl* cu, int gi) {
         dt = wp<T>(cu->dt[gi], cu->dt_f[gi]);
         rs = cu->reset[gi] != 0;
         f = wp<T>(cu->f, cu->f_f);
@@ -567,115 +504,142 @@ __global__ void __launch_bounds__(BLOCK, (integrate_minb<T, D, MODE>()))
             f = wp<T>(cu->gf[gi], cu->gf_f[gi]);
             eps = wp<T>(cu->geps[gi], cu->geps_f[gi]);
         }
-        const Vec4<T> ai = s.A[k];
-        const T api[3] = {ai.x, ai.y, ai.z};
-        for (int a = 0; a < 3; ++a) {
-            const T vp = rs ? T(0) : f * v[a];
-            vt[a] = vp + dt * (api[a] - eps * vp);
-        }
-        if (MODE != 2 && di < D) {
-            T xi[3];
-            pos_t<T, D>(g, c, o3, xi);
-            feature_tangent<T>(dom.f[gi], xi, tg);
-        }
     }
-    if (MODE != 2 && p.visc > 0.0 && !done) {
-        const T kappa = wp<T>(p.kappa, p.kappa_f), hk = T(0.5) * kappa, visc = wp<T>(p.visc, p.visc_f);
-        T hid, hi2d;
-        hpow(hi, di > 0 ? di : 1, hid, hi2d);
-        const T eta_i = visc * kappa * hi * t_sqrt(vt[0] * vt[0] + vt[1] * vt[1] + vt[2] * vt[2]) * fast_rcp(hid);
-        // the pair's kernel factor of Eq. 7, (rho_i^-2 + rho_j^-2) W'(r, h_ij) / r (the pressure
-        // pass hands it over with the pair; computed here for the pairs of an overflowed list)
-        auto kfac = [&](T hj, T r) {
-            T hjd, hj2d;
-            hpow(hj, di, hjd, hj2d);
-            const T invR = fast_rcp(hk * (hi + hj));
-            const T q = r * invR;
-            const T t = T(1) - q;
-            const T dW = wendland_alpha<T>(di, invR) * (T(-20) * q * t * t * t) * invR;
-            return (hi2d + hj2d) * dW * fast_rcp(r);
-        };
-        // one same-group pair (its kernel factor kv, its a_p and (v, h) loaded): the viscous term
-        // of Eq. 7
-        auto pair = [&](const Vec4<T>& aj, const Vec4<T>& vhj, T kv) {
-            const T hj = vhj.w;
-            const T apj[3] = {aj.x, aj.y, aj.z};
-            const T vj3[3] = {vhj.x, vhj.y, vhj.z};
-            T vtj[3] = {T(0), T(0), T(0)};
-            for (int a = 0; a < D; ++a) {
-                const T vp = rs ? T(0) : f * vj3[a];
-                vtj[a] = vp + dt * (apj[a] - eps * vp);
-            }
-            T hjd, hj2d;
-            hpow(hj, di, hjd, hj2d);
-            const T eta_j = visc * kappa * hj * t_sqrt(vtj[0] * vtj[0] + vtj[1] * vtj[1] + vtj[2] * vtj[2]) *
-                            fast_rcp(hjd);
-            const T es = eta_i + eta_j;
-            if (!(es > T(0))) return;
-            const T eb = T(2) * eta_i * eta_j / es;
-            const T coef = eb * kv;
-            for (int a = 0; a < D; ++a) av[a] += coef * (vt[a] - vtj[a]);
-        };
-        // the pairs the pressure pass found (list), or the cell walk where the list overflowed
-        constexpr int VCAP = Vcap<D>::v;
-        // this lane's columns of the hand-over list: pressure-pass lanes sub + t LPP, t < NCOL
-        const int NL = s.n * LPI, lg0 = k * LPI + (int)(threadIdx.x % LPP);
-        int vc[NCOL];
-        int over = 0;
-#pragma unroll
-        for (int t = 0; t < NCOL; ++t) {
-            vc[t] = moving ? s.vcnt[lg0 + t * LPP] : 0;
-            over |= vc[t] > VCAP ? 1 : 0;
-        }
-        const bool ov = sub_sum<LPP>(over) != 0;   // overflow in any column of the particle
-        if (moving && !ov)
-#pragma unroll
-            for (int t = 0; t < NCOL; ++t) {
-                const int lg = lg0 + t * LPP;
-                // SPH_VISC_BATCH entries at a time: their loads are all issued before the first use
-                for (int e0 = 0; e0 < vc[t]; e0 += SPH_VISC_BATCH) {
-                    constexpr int U = SPH_VISC_BATCH;
-                    int jj[U];
-                    T rr[U];
-                    Vec4<T> aj[U], vhj[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (e0 + u < vc[t]) {
-                            jj[u] = s.vj[(size_t)(e0 + u) * NL + lg];
-                            rr[u] = s.vr[(size_t)(e0 + u) * NL + lg];
-                        }
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (e0 + u < vc[t]) {
-                            aj[u] = s.A[jj[u]];
-                            vhj[u] = s.VH[jj[u]];
-                        }
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (e0 + u < vc[t]) pair(aj[u], vhj[u], rr[u]);
-                }
-            }
-        int li = 0, ci[3] = {0, 0, 0};
-        if (moving && ov) own_cell<T, D>(g, s, k, hi, li, ci);
-        walk_sub<T, D, LPP, BUF_CAP>(
-            g, s.cell_start, s.occ, s.n, s.P, s.Ms, sbuf + threadIdx.x, moving && ov, li, ci, offi, hi, kappa,
-            [&](int j, const T*, T r2, T hj, unsigned mj) -> bool {
-                return meta_group(mj) == gi && j != k && r2 < pair_rc2(hi, hj, hk) && r2 > T(0);
-            },
-            [&](int j, const T*, T r2, T hj, unsigned, const T*, int, int, int, int) {
-                pair(s.A[j], s.VH[j], kfac(hj, r2 * fast_rsqrt(r2)));
-            });
-        for (int a = 0; a < D; ++a) av[a] = sub_sum<LPP>(av[a]);
-        if (moving) tangent_map<T>(di, D, tg, av);
+};
+
+// (v~, eta) of a moving particle of dimension di from its (a_p, V~) and (v, h) records
+template <typename T>
+__device__ __forceinline__ Vec4<T> predicted(const Params& p, const StepOf<T>& st, const Vec4<T>& a, const Vec4<T>& vh, int di) {
+    const T v[3] = {vh.x, vh.y, vh.z}, ap[3] = {a.x, a.y, a.z};
+    T vt[3];
+    for (int c = 0; c < 3; ++c) {
+        const T vp = st.rs ? T(0) : st.f * v[c];
+        vt[c] = vp + st.dt * (ap[c] - st.eps * vp);
     }
-    if constexpr (MODE == 1) {
-        if (lead && moving)
-            for (int a = 0; a < D; ++a) o.V[a][k] = av[a];
+    T hd, h2d;
+    hpow(vh.w, di, hd, h2d);
+    Vec4<T> q;
+    q.x = vt[0];
+    q.y = vt[1];
+    q.z = vt[2];
+    q.w = wp<T>(p.visc, p.visc_f) * wp<T>(p.kappa, p.kappa_f) * vh.w *
+          t_sqrt(vt[0] * vt[0] + vt[1] * vt[1] + vt[2] * vt[2]) * fast_rcp(hd);
+    return q;
+}
+
+template <typename T, int D, bool ONE>
+__global__ void __launch_bounds__(BLOCK) k_predict(State<T> s, One one, const Ctrl* use, int cls) {
+    dep_launch();
+    dep_wait();
+    const int k = blockIdx.x * BLOCK + threadIdx.x;
+    if (k >= s.n) return;
+    const int inst = ONE ? 0 : inst_of(s, k);
+    if (!live(s, inst, k)) return;
+    const Params& p = ONE ? one.p : s.params[inst];
+    const Vec4<T> vh = s.VH[k], a = s.A[k];
+    const unsigned mi = slot_meta<T, D>(s, k);
+    const int gi = meta_group(mi), di = meta_dim(mi);
+    if (moves(p, use + inst, gi, di, cls, D)) s.A[k] = predicted<T>(p, StepOf<T>(p, use + inst, gi), a, vh, di);
+}
+
+// 2 a b / (a + b) for a, b >= 0 (0 where the sum is 0)
+template <typename T> __device__ __forceinline__ T harmonic(T a, T b) {
+    const T s = a + b;
+    return s > T(0) ? T(2) * a * b / s : T(0);
+}
+
+// the viscous term of Eq. 7 of a pair: me, q the two particles' (v~, eta), kv the kernel factor
+template <typename T, int D> __device__ __forceinline__ void visc_pair(const Vec4<T>& me, const Vec4<T>& q, T kv, T av[3]) {
+    const T c = harmonic(me.w, q.w) * kv;
+    av[0] += c * (me.x - q.x);
+    av[1] += c * (me.y - q.y);
+    if (D == 3) av[2] += c * (me.z - q.z);
+}
+
+// the viscous sums of the warp's particles whose list overflowed (over), from a second search; all
+// lanes call this together (not inlined: rarely needed, and its registers would weigh on k_visc)
+template <typename T, int D, bool FUSED>
+__device__ __noinline__ void visc_again(const State<T>& s, const Grid& g, const Params& p, const Ctrl* cu,
+                                        SearchWarp<32 / Lpp<D>::v>& ww, int lane, int k0, bool over, Vec4<T> me, T* av) {
+    constexpr int LPP = Lpp<D>::v, CL = 32 / LPP;
+    const int k = k0 + lane / LPP, sub = lane % LPP;
+    const Meta<D>* const Ms = meta_words<D>(s);
+    const T hk = T(0.5) * wp<T>(p.kappa, p.kappa_f);
+    T offi[3] = {T(0), T(0), T(0)}, hi = T(1), sum[3] = {T(0), T(0), T(0)}, hid, hi2d;
+    int li = 0, ci[3] = {0, 0, 0}, Pi[3], gi = 0, di = 1;
+    if (over) {
+        Meta<D> wi;
+        Rec<T, D>::load(s.P, Ms, k, offi, hi, wi);
+        own_cell<T, D>(g, s, k, hi, li, ci);
+        gi = meta_group(MetaWord<D>::meta(wi));
+        di = meta_dim(MetaWord<D>::meta(wi));
+    }
+    hpow(hi, di, hid, hi2d);
+    for (int a = 0; a < 3; ++a) Pi[a] = ci[a] << li;
+    unsigned long long none = 0;
+    warp_search<T, D, CL, true>(
+        g, s, ww, lane, k0, over, over ? s.F[k] : make_float4(0.0f, 0.0f, 0.0f, 0.0f), li, ci, none, [&](int m_) {
+            for (int t = sub; t < m_; t += LPP) {
+                const int j = s.vj[(size_t)k * ListShape<D>::ROW + t];
+                T offj[3], hj, dx[3], hjd, hj2d;
+                Meta<D> w;
+                int m[3];
+                Rec<T, D>::load(s.P, Ms, j, offj, hj, w);
+                MetaWord<D>::rel(w, Pi, m);
+                const T r2 = pair_dx<T, D>(offi, offj, m, (T)g.c0, dx);
+                if (meta_group(MetaWord<D>::meta(w)) != gi || !(r2 < pair_rc2(hi, hj, hk)) || !(r2 > T(0))) continue;
+                hpow(hj, di, hjd, hj2d);
+                const Vec4<T> q = FUSED ? predicted<T>(p, StepOf<T>(p, cu, gi), s.A[j], s.VH[j], di) : s.A[j];
+                visc_pair<T, D>(me, q,
+                                (hi2d + hj2d) * wendland_slope<T>(di, root_of(r2), fast_rcp(hk * (hi + hj))), sum);
+            }
+        });
+    for (int a = 0; a < 3; ++a) av[a] += sum[a];
+}
+
+// one particle moved (slot k of instance inst; padding slots are copied through unchanged)
+template <typename T, int D, bool FUSED>
+__device__ __forceinline__ void update_one(const State<T>& s, const Grid& g, const Params& p, const Ctrl* cu, const Out<T>& o,
+                                           int inst, int k, int cls, const T* av_in) {
+    Ctrl* const ctrl = s.ctrls + inst;
+    const Domain& dom = s.doms[inst];
+    if (!live(s, inst, k)) {   // padding: keep the slot as it is
+        const Vec4<T> vh = s.VH[k];
+        const T vv[3] = {vh.x, vh.y, vh.z};
+        for (int a = 0; a < D; ++a) {
+            o.C[a][k] = s.Cs[a][k];
+            o.O[a][k] = s.Os[a][k];
+            o.V[a][k] = vv[a];
+            if (o.av[a]) o.av[a][k] = T(0);
+        }
+        o.H[k] = vh.w;
+        o.G[k] = 0u;
+        o.ID[k] = s.IDs[k];
+        if (o.K) {   // the next rebuild's key: the instance's dummy cell
+            o.K[k] = g.base[MAXL];
+            atomicAdd(o.count + g.base[MAXL], 1);
+        }
         return;
     }
-    if (MODE == 2 && moving)
-        for (int a = 0; a < D; ++a) av[a] = o.V[a][k];
-    if (!lead) return;
+    const Vec4<T> vh = s.VH[k];
+    const T hi = vh.w;
+    const unsigned mi = slot_meta<T, D>(s, k);
+    int c[3] = {0, 0, 0};            // stored position: finest cell + offset
+    T o3[3] = {T(0), T(0), T(0)};
+    T v[3] = {vh.x, vh.y, vh.z};
+    for (int a = 0; a < D; ++a) {
+        c[a] = s.Cs[a][k];
+        o3[a] = s.Os[a][k];
+    }
+    const int gi = meta_group(mi), di = meta_dim(mi);
+    const bool moving = moves(p, cu, gi, di, cls, D);
+    T av[3] = {T(0), T(0), T(0)}, vt[3] = {T(0), T(0), T(0)}, hnew = hi, dt = T(0);
+    if (moving) {
+        dt = wp<T>(cu->dt[gi], cu->dt_f[gi]);
+        const Vec4<T> q = FUSED ? predicted<T>(p, StepOf<T>(p, cu, gi), s.A[k], vh, di) : s.A[k];
+        vt[0] = q.x, vt[1] = q.y, vt[2] = q.z;
+        for (int a = 0; a < D; ++a) av[a] = FUSED ? av_in[a] : o.V[a][k];
+    }
     if (moving) {
         const Feat& fi = dom.f[gi];
         // x+ = x + dt v+, advanced on the offset and re-normalised into the finest cell
@@ -735,7 +699,6 @@ __global__ void __launch_bounds__(BLOCK, (integrate_minb<T, D, MODE>()))
         for (int a = 0; a < D; ++a) fin = fin && isfinite(o3[a]) && isfinite(v[a]);
         if (!fin) atomicOr(&ctrl->status, ST_NONFINITE);
     }
-    if (!inrange) return;
     if (di == 0) v[0] = v[1] = v[2] = T(0);
     for (int a = 0; a < D; ++a) {
         o.C[a][k] = c[a];
@@ -756,6 +719,108 @@ __global__ void __launch_bounds__(BLOCK, (integrate_minb<T, D, MODE>()))
     }
 }
 
+
+template <typename T, int D, bool ONE, bool FUSED>
+__global__ void __launch_bounds__(BLOCK, (FUSED || sizeof(T) == 8 ? 4 : (D == 2 ? SPH_VISC_MINB_2D : SPH_VISC_MINB_3D)))
+    k_visc(const __grid_constant__ State<T> s, const __grid_constant__ One one, const Ctrl* use, Out<T> o, int cls) {
+    dep_launch();
+    dep_wait();
+    constexpr int LPP = Lpp<D>::v, CL = 32 / LPP, U = LISTU;
+    __shared__ SearchWarp<CL> ww[BLOCK / 32];
+    __shared__ Grid gsh;
+    __shared__ Params psh;
+    const int lane = lane_id(), sub = lane % LPP;
+    const int k0 = (blockIdx.x * (BLOCK / 32) + (threadIdx.x >> 5)) * CL, k = k0 + lane / LPP;
+    const int inst = ONE ? 0 : __ldg(s.chunk_inst + k0 / CHUNK);
+    const Ctrl* const cu = use + inst;
+    if (!ONE) {
+        block_copy(&gsh, s.grids + inst);
+        block_copy(&psh, s.params + inst);
+        __syncthreads();
+    }
+    const Grid& g = ONE ? one.g : gsh;
+    const Params& p = ONE ? one.p : psh;
+    const bool inrange = k < s.n && live(s, inst, k);
+    const unsigned mi = inrange ? slot_meta<T, D>(s, k) : 0u;
+    const int gi = meta_group(mi), di = meta_dim(mi);
+    const bool moving = inrange && moves(p, cu, gi, di, cls, D);
+    T av[3] = {T(0), T(0), T(0)};
+    const StepOf<T> st(p, cu, moving ? gi : 0);
+    if (p.visc > 0.0) {
+        Vec4<T> me;
+        me.x = me.y = me.z = me.w = T(0);
+        if (moving) me = FUSED ? predicted<T>(p, st, s.A[k], s.VH[k], di) : s.A[k];
+        const int n = moving ? s.vcnt[k] : 0;
+        const bool over = moving && list_overflowed<T, D>(s, k, n);
+        const unsigned long long xid = n > ListShape<D>::ROW ? s.xid[k] : 0ull;
+        if (!over)
+            for (int t = sub * U; t < n; t += LPP * U) {
+                int jj[U];
+                T kv[U];
+                Vec4<T> q[U], vh[FUSED ? U : 1];
+                const size_t e = list_entry<T, D>(s, k, t, xid);
+                list_load(s.vj + e, jj);
+                list_load(s.vr + e, kv);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (t + u >= n) kv[u] = T(0), jj[u] = k;
+                    q[u] = s.A[jj[u]];
+                    if (FUSED) vh[u] = s.VH[jj[u]];
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (kv[u] != T(0))
+                        visc_pair<T, D>(me, FUSED ? predicted<T>(p, st, q[u], vh[FUSED ? u : 0], di) : q[u], kv[u], av);
+            }
+        if (__any_sync(0xffffffffu, over)) visc_again<T, D, FUSED>(s, g, p, cu, ww[threadIdx.x >> 5], lane, k0, over, me, av);
+        for (int a = 0; a < D; ++a) av[a] = sub_sum<LPP>(av[a]);
+        if (moving && di < D) {
+            T xi[3] = {T(0), T(0), T(0)}, o3[3] = {T(0), T(0), T(0)}, tg[3];
+            int c[3] = {0, 0, 0};
+            for (int a = 0; a < D; ++a) {
+                c[a] = s.Cs[a][k];
+                o3[a] = s.Os[a][k];
+            }
+            pos_t<T, D>(g, c, o3, xi);
+            const Domain& dom = s.doms[inst];
+            feature_tangent<T>(dom.f[gi], xi, tg);
+            tangent_map<T>(di, D, tg, av);
+        }
+    }
+    if constexpr (FUSED) {   // the block's first warp moves its particles, one per lane
+        constexpr int PB = BLOCK / LPP;
+        static_assert(PB == 32, "one warp's worth of particles per block");
+        __shared__ T sh_av[PB][3];
+        if (sub == 0)
+            for (int a = 0; a < D; ++a) sh_av[threadIdx.x / LPP][a] = av[a];
+        if (o.K) reset_scan_state(s);   // this kernel produces the next scan's histogram
+        __syncthreads();
+        const int ku = blockIdx.x * PB + threadIdx.x;
+        if (threadIdx.x < PB && ku < s.n) update_one<T, D, true>(s, g, p, cu, o, inst, ku, cls, sh_av[threadIdx.x]);
+    } else if (moving && sub == 0) {
+        for (int a = 0; a < D; ++a) o.V[a][k] = av[a];
+    }
+}
+
+template <typename T, int D, bool ONE>
+__global__ void __launch_bounds__(BLOCK, (sizeof(T) == 4 ? SPH_UPDATE_MINB : 4))
+    k_update(State<T> s, One one, const Ctrl* use, Out<T> o, int cls) {
+    dep_launch();
+    dep_wait();
+    __shared__ Grid gsh;
+    __shared__ Params psh;
+    const int inst = ONE ? 0 : __ldg(s.chunk_inst + (blockIdx.x * BLOCK) / CHUNK);
+    if (!ONE) {
+        block_copy(&gsh, s.grids + inst);
+        block_copy(&psh, s.params + inst);
+        __syncthreads();
+    }
+    if (o.K) reset_scan_state(s);   // this kernel produces the next scan's histogram
+    const int k = blockIdx.x * BLOCK + threadIdx.x;
+    if (k < s.n) update_one<T, D, false>(s, ONE ? one.g : gsh, ONE ? one.p : psh, use + inst, o, inst, k, cls, nullptr);
+}
+
+
 template <typename T, int D> void launch_control(const State<T>& s, const One* one, cudaStream_t st, bool pdl, int cls) {
     if (one) launch_k(k_control<T, D, true>, s.NI, CTL_THREADS, st, pdl, s, *one, cls);
     else launch_k(k_control<T, D, false>, s.NI, CTL_THREADS, st, pdl, s, One(), cls);
@@ -763,18 +828,19 @@ template <typename T, int D> void launch_control(const State<T>& s, const One* o
 template <typename T, int D>
 void launch_integrate(const State<T>& s, const One* one, const Ctrl* use, const Out<T>& o, cudaStream_t st,
                       bool pdl, int cls) {
-    const int nb = div_up((long long)s.n * ILpp<D>::v, BLOCK);
-    if (D == 2 ? SPH_SPLIT_INTEGRATE_2D : SPH_SPLIT_INTEGRATE_3D) {   // viscous sum, then update
-        const int nu = div_up((long long)s.n, BLOCK);
-        if (one) {
-            launch_k(k_integrate<T, D, true, 1>, nb, BLOCK, st, pdl, s, *one, use, o, cls);
-            launch_k(k_integrate<T, D, true, 2>, nu, BLOCK, st, pdl, s, *one, use, o, cls);
-        } else {
-            launch_k(k_integrate<T, D, false, 1>, nb, BLOCK, st, pdl, s, One(), use, o, cls);
-            launch_k(k_integrate<T, D, false, 2>, nu, BLOCK, st, pdl, s, One(), use, o, cls);
-        }
-    } else if (one) launch_k(k_integrate<T, D, true, 0>, nb, BLOCK, st, pdl, s, *one, use, o, cls);
-    else launch_k(k_integrate<T, D, false, 0>, nb, BLOCK, st, pdl, s, One(), use, o, cls);
+    const int nb = div_up((long long)s.n * Lpp<D>::v, BLOCK), nu = div_up((long long)s.n, BLOCK);
+    if (sizeof(T) == 4 && s.n <= (D == 2 ? SPH_FUSED_MOST_2D : SPH_FUSED_MOST_3D)) {
+        if (one) launch_k(k_visc<T, D, true, true>, nb, BLOCK, st, pdl, s, *one, use, o, cls);
+        else launch_k(k_visc<T, D, false, true>, nb, BLOCK, st, pdl, s, One(), use, o, cls);
+    } else if (one) {
+        launch_k(k_predict<T, D, true>, nu, BLOCK, st, pdl, s, *one, use, cls);
+        launch_k(k_visc<T, D, true, false>, nb, BLOCK, st, true, s, *one, use, o, cls);
+        launch_k(k_update<T, D, true>, nu, BLOCK, st, true, s, *one, use, o, cls);
+    } else {
+        launch_k(k_predict<T, D, false>, nu, BLOCK, st, pdl, s, One(), use, cls);
+        launch_k(k_visc<T, D, false, false>, nb, BLOCK, st, true, s, One(), use, o, cls);
+        launch_k(k_update<T, D, false>, nu, BLOCK, st, true, s, One(), use, o, cls);
+    }
 }
 
 #define SPH_INST(T, D)                                                      \

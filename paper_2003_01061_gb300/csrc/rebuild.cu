@@ -258,6 +258,7 @@ template <typename T, int D, bool ONE> __global__ void __launch_bounds__(BLOCK) 
     dep_wait();
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= s.n) return;
+    if (k % CHUNK == 0) s.xcnt[k / CHUNK] = 0;   // the chunk's list blocks (search)
     int i = s.perm[k];
     const int key = s.Ks[k];
     if ((unsigned)i >= (unsigned)s.n || (unsigned)key >= (unsigned)s.ncell) {
@@ -313,8 +314,19 @@ template <typename T, int D, bool ONE> __global__ void __launch_bounds__(BLOCK) 
     int cell[3];
     T off[3];
     level_repr<T, D>(g, l, c, o, cell, off);
-    Rec<T, D>::store(s.P, s.Ms, k, off, h, (meta & 255u) | ((unsigned)cell[0] << 8));
-    if (s.occ) {   // the largest h of the particle's level in the occupancy cell holding it
+    const int corner[3] = {cell[0] << l, cell[1] << l, cell[2] << l};
+    // search record: position and half support in finest cells; the half support is widened by
+    // more than the rounding of h, of the support and of the search's comparison
+    const Params& p = ONE ? one.p : s.params[inst];
+    const float ic0 = 1.0f / g.c0;
+    float4 f;
+    f.x = fmaf((float)off[0], ic0, (float)corner[0]);
+    f.y = fmaf((float)off[1], ic0, (float)corner[1]);
+    f.z = D == 3 ? fmaf((float)off[2], ic0, (float)corner[2]) : 0.0f;
+    f.w = (0.5f * p.kappa_f * ic0 * (1.0f + 0x1p-12f)) * (float)h;
+    s.F[k] = f;
+    Rec<T, D>::store(s.P, meta_words<D>(s), k, off, h, MetaWord<D>::make(meta, corner));
+    if (s.occ) {   // the largest half support of the particle's level in the occupancy cell holding it
         const int sh = g.osh;
         int ct[3] = {0, 0, 0};
         for (int a = 0; a < D; ++a) ct[a] = min((cell[a] << l) >> sh, g.od[a] - 1);
@@ -322,7 +334,7 @@ template <typename T, int D, bool ONE> __global__ void __launch_bounds__(BLOCK) 
         // sorted neighbours share the cell and the level: one atomic per distinct pair in the
         // warp (positive floats order as their bits)
         const unsigned peers = __match_any_sync(__activemask(), ((unsigned long long)w << 4) | (unsigned)l);
-        const unsigned hbits = __reduce_max_sync(peers, __float_as_uint(float_up<T>(h)));
+        const unsigned hbits = __reduce_max_sync(peers, __float_as_uint(f.w));
         if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicMax(s.occ + (size_t)w * OCCW + l, hbits);
     }
 }

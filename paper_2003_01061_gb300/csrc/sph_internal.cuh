@@ -43,6 +43,7 @@ template <typename T> struct State {
     int* IDs;
     int* Ks;
     Vec4<T>* P;
+    float4* F;         // search records: position and kappa h / 2 in finest cells (padding: stale)
     Vec4<T>* A;
     // rebuild scratch: per-cell counts (also the scatter cursors), cell starts, scan block
     // sums, and the sorted-slot -> stored-index permutation
@@ -57,22 +58,23 @@ template <typename T> struct State {
     int* perm;         // slot -> stored index as left by the scatter (unordered inside a cell)
     int* sperm;        // slot -> stored index, stable (ordered inside a cell; written by the gather)
     int ncell;         // total keys (all instances' cells and dummy cells)
-    // per occupancy cell, OCCW words: per level the largest h of its particles in the cell
-    // (float bits, 0 for none; built by the gather)
+    // per occupancy cell, OCCW words: per level the largest half support (F's w) of its
+    // particles in the cell (float bits, 0 for none; built by the gather)
     unsigned* occ;
     int nocc;
-    // same-group pairs found by the pressure pass, handed to the viscous pass: for lane
-    // g = k*LPP + r of particle k, entry c is (vj, vr)[c * n*LPP + g] (index, and the pair's
-    // kernel factor of Eq. 7, (rho_i^-2 + rho_j^-2) W'(r, h_ij) / r);
-    // vcnt[g] counts them (> VCAP: the list overflowed and the viscous pass walks the cells)
+    // neighbour lists (ListShape): the rows by slot, then, from entry xbase, the blocks by chunk;
+    // per entry the candidate (search) and the pair's kernel factor of Eq. 7,
+    // (rho_i^-2 + rho_j^-2) W'(r, h_ij) / r (pressure pass; 0: no pair of the viscous sum); per slot
+    // the number of candidates and, for a list longer than its row, its blocks (a byte each); per
+    // chunk the number of blocks asked for
     int* vj;
     T* vr;
     int* vcnt;
-    // per-block, per-group partial sums of V~ (sample steps); nblk = blocks of the pair passes.
-    // The last pressure-pass block of every chunk of CHUNK slots (counted in pticket) adds the
-    // chunk's block rows in block order into partials2 [chunk][MAXF], which the controller reads
-    double* partials;
-    int nblk;
+    unsigned long long* xid;
+    int* xcnt;
+    size_t xbase;
+    // sums of V~ per chunk of CHUNK slots and group (sample steps), [chunk][MAXF]: written by the
+    // chunk's last pressure-pass warp (counted in pticket), read by the controller
     double* partials2;
     int* pticket;
 };
@@ -97,71 +99,79 @@ template <typename T> struct Out {
     int* count;        // ... and per-cell histogram, so that the next step needs no hash pass
 };
 
-// (measured with the 2.6h support: 12 / 20 / 24 make the whole 2D step 22 % slower / 1 % slower /
-// 5 % slower than 16, and the 1.2M cube's 33 % / 2 % / 11 %)
-// the pressure pass's per-block Eq. 24 minima and V~ partial sums in the memory of its
-// candidate buffers once the walk is done (1) or in arrays of their own (0) (measured: 3D
-// pressure pass on the 1.2M cube 3.36 ms against 3.42, 2D on the 120k disk 80.1 us against 79.0)
-#ifndef SPH_ALIAS_TAIL_2D
-#define SPH_ALIAS_TAIL_2D 0
-#endif
-#ifndef SPH_ALIAS_TAIL_3D
-#define SPH_ALIAS_TAIL_3D 1
-#endif
-#ifndef SPH_BUF_CAP
-#define SPH_BUF_CAP 16
-#endif
-constexpr int BUF_CAP = SPH_BUF_CAP;   // kept candidates per lane between flushes of the walk (shared memory)
-// lanes per particle in the pair passes (measured with a 2.6h support, 5 steps after the start,
-// whole step in ms for disks of 1k / 20k / 120k / 1M particles: 2 lanes 0.134 / 0.123 / 0.183 /
-// 0.829, 4 lanes with 64 hand-over slots 0.096 / 0.093 / 0.153 / 0.828; 1 lane 1.7-2.5x slower;
-// cubes of 20k / 200k / 1.2M: 8 lanes 0.229 / 1.018 / 4.92, 4 lanes 0.50 / 1.79 / 9.44, 16 lanes
-// 0.48 / 1.60 / 7.54, 16 faster only at 1k (0.166 against 0.199); fewer lanes repeat less of
-// the per-particle stencil work, more lanes balance the candidates)
+// lanes per particle in the pair passes over the neighbour lists (measured, whole step in us with
+// 4 / 8 / 16: 20k disk 76 / 78 / 84, 120k disk 144 / 159 / 206, 83k cube 320 / 328 / 363, 300k cube
+// 706 / 778 / 935; a result must not depend on the batch, so the number is the same at every size)
 #ifndef SPH_LPP_2D
 #define SPH_LPP_2D 4
 #endif
 #ifndef SPH_LPP_3D
-#define SPH_LPP_3D 8
+#define SPH_LPP_3D 4
 #endif
 template <int D> struct Lpp {
     static constexpr int v = D == 2 ? SPH_LPP_2D : SPH_LPP_3D;
 };
-// same-group pair slots per particle (SPH_VCAP_2D/3D) and per lane (Vcap) in the
-// pressure-to-viscous hand-over list (measured with a 2.6h support, whose overflowing particles
-// walk the cells again: in 2D with 4 lanes per particle 64 slots make the 120k disk's step 5 %
-// faster than 48, 96 no faster; in 3D 192 slots are 4.5x faster than 96 on the viscous pass,
-// 128 make the 1.2M cube's step 11 % slower and 256 no faster)
-#ifndef SPH_VCAP_2D
-#define SPH_VCAP_2D 64
-#endif
-#ifndef SPH_VCAP_3D
-#define SPH_VCAP_3D 192
-#endif
-template <int D> struct Vcap {
-    static constexpr int v = D == 2 ? SPH_VCAP_2D / Lpp<2>::v : SPH_VCAP_3D / Lpp<3>::v;
+// Neighbour lists: the candidates within the larger of a particle's own and the pair's radius,
+// itself included, about 24 in 2D and 80 in 3D.  A particle has a row of ROW entries; a longer list
+// goes on in up to XMAX blocks of XB entries, taken from the NXB blocks of its chunk of slots
+// (coarse particles beside much finer ones: a few per mille of a graded 3D mesh).  A list that
+// needs more, or any list with blocks in a chunk that ran out of them, counts as overflowed (which
+// lists got blocks there depends on timing, whether the chunk ran out does not): the pair passes
+// search those particles' neighbours again.
+template <int D> struct ListShape;
+template <> struct ListShape<2> {
+    static constexpr int ROW = 48, XB = 32, NXB = 64;
 };
-// lanes per particle in the viscous pass; each lane reads Lpp/ILpp of the pressure pass's
-// hand-over columns, and the list-overflow fallback walks with ILpp lanes (measured: one lane
-// in 2D, 2 % faster than 2; in 3D with the 2.6h support and 192 list slots per particle, on the
-// 1.2M cube after 5 steps, 2 lanes make the pass 0.854 ms against 1.177 ms with one lane (27 %
-// faster; with 5 blocks per SM 0.891 ms), and 3 entries fetched together instead of 2 are 74 %
-// slower)
-#ifndef SPH_ILPP_2D
-#define SPH_ILPP_2D 1
-#endif
-#ifndef SPH_ILPP_3D
-#define SPH_ILPP_3D 2
-#endif
-template <int D> struct ILpp {
-    static constexpr int v = D == 2 ? SPH_ILPP_2D : SPH_ILPP_3D;
+template <> struct ListShape<3> {
+    static constexpr int ROW = 128, XB = 64, NXB = 128;
 };
-static_assert(CHUNK % (BLOCK / Lpp<2>::v) == 0 && CHUNK % (BLOCK / Lpp<3>::v) == 0 &&
-                  CHUNK % (BLOCK / ILpp<2>::v) == 0 && CHUNK % (BLOCK / ILpp<3>::v) == 0,
+constexpr int XMAX = 8;
+template <int D> constexpr int list_most() { return ListShape<D>::ROW + XMAX * ListShape<D>::XB; }
+// entries per slot, blocks included
+template <int D> constexpr int list_entries() {
+    return ListShape<D>::ROW + ListShape<D>::XB * ListShape<D>::NXB / CHUNK;
+}
+// consecutive list entries per lane and turn of the pair passes: their loads are in flight together
+// (measured on the 1.2M cube: 4 against 2 viscous sum and update 339 us against 468)
+#ifndef SPH_LISTU
+#define SPH_LISTU 4
+#endif
+constexpr int LISTU = SPH_LISTU;
+// particles searched by one warp: 2, 4, 8 or 16 by the slots of the batch (up to N2, N4, N8 slots).
+// A warp searching for more particles reads the cells around them once for all, one searching for
+// fewer is done sooner, which counts while the GPU is not full.  The lists do not depend on it.
+// Measured, search and pressure pass in us with 2 / 4 / 8 / 16: a 26k ball in three passes (whole
+// step) 376 / 437 / 640 / 826; a 20k disk 33 / 29 / 38 / 55; 120k disk 106 / 76 / 66 / 79; 1M disk
+// - / - / 430 / 404; 83k cube 189 / 149 / 137 / 146; 300k cube 671 / 498 / 472 / -; 1.2M cube
+// 2447 / - / 1451 / 1408.
+#ifndef SPH_SEARCH_CL
+#define SPH_SEARCH_CL 0
+#endif
+#ifndef SPH_SEARCH_N2
+#define SPH_SEARCH_N2 (D == 3 ? 32768 : 0)
+#endif
+#ifndef SPH_SEARCH_N4
+#define SPH_SEARCH_N4 65536
+#endif
+#ifndef SPH_SEARCH_N8
+#define SPH_SEARCH_N8 524288
+#endif
+// most slots of a batch whose prediction, viscous sum and update run as one kernel (FP32 build).
+// Measured, one kernel against three, us per step: the 2.6k square 48.6 against 52.2, a 20k disk
+// 77.2 against 79.8, a 120k disk 156.3 against 138.9; 3D, a 26k ball in three passes 372 against
+// 363.  In FP64 the neighbours' predictions cost more than the launches (2.9k square 116 against 110).
+#ifndef SPH_FUSED_MOST_2D
+#define SPH_FUSED_MOST_2D 32768
+#endif
+#ifndef SPH_FUSED_MOST_3D
+#define SPH_FUSED_MOST_3D 8192
+#endif
+// resident one-warp blocks per SM asked of the compiler for the search (measured, 8 particles per
+// warp: 32 blocks at 64 registers with a few spills against 24 at 80, search and pressure pass of
+// the 1M disk 430 us against 461, of the 1.2M cube 1451 against 1552)
+constexpr int search_minb(int cl) { return cl == 16 ? 28 : 32; }
+static_assert(CHUNK % (BLOCK / Lpp<2>::v) == 0 && CHUNK % (BLOCK / Lpp<3>::v) == 0,
               "a pair-pass block must lie in one chunk");
-static_assert(Lpp<2>::v % ILpp<2>::v == 0 && Lpp<3>::v % ILpp<3>::v == 0,
-              "the viscous lanes split the pressure pass's columns evenly");
-
 // 3D occupancy cells finer than the cells-per-support top-level cells by 2^SPH_OCC_FINER per axis
 // (measured on the 3D cube: 1 and 2 make the pressure pass 5 % and 21 % slower than 0; with the
 // search radius from the cells' largest h, 6 % and 16 %)
@@ -169,46 +179,28 @@ static_assert(Lpp<2>::v % ILpp<2>::v == 0 && Lpp<3>::v % ILpp<3>::v == 0,
 #define SPH_OCC_FINER 0
 #endif
 
-// minimum resident blocks per SM asked of the compiler for the two pair passes (FP32 build;
-// the FP64 build asks for 4): it bounds the registers per thread, trading spills for occupancy
-// (measured on the pressure pass: 10 and 12 spill and are 17 % and 40 % slower than 8; with
-// the 2.6h support and 8 lanes per particle in 3D, on a 1.2M cube, 5 / 6 / 7 / 9 / 10 were
-// 24 / 13 / 8 / 10 / 46 % slower than 8 although 8 spills a few words in the batched form,
-// and 9 in 2D 4 % slower; on the viscous pass with one lane per particle 7 is 3 % faster than
-// 8 in 2D, and 6 is 5 % faster than 7 in 3D but 26 % slower in 2D; again with the 2.6h support:
-// 2D 6 / 8 30 % / 3 % slower than 7, 3D 5 2 % faster than 6 on the pass (0.3 % on the step)
-// and 7 12 % slower)
+// minimum resident blocks per SM asked of the compiler for the pair passes: it bounds the registers
+// per thread, trading spills for warps in flight (measured, search and pressure pass in us: 2D, 1M
+// disk, 5 / 6 / 7 / 8 blocks 499 / 472 / 443 / 428; 3D, 1.2M cube, 5 / 6 / 7 / 8 blocks 1541 / 1499 /
+// 1504 / 1595; FP64, 40k cube, 4 / 6 blocks 791 / 990; viscous sum and update: 1M disk 6 / 8 / 10 /
+// 12 blocks 219 / 201 / 182 / 172, 1.2M cube 8 / 10 / 12 blocks 392 / 362 / 439)
 #ifndef SPH_INTERACT_MINB
 #define SPH_INTERACT_MINB 8
 #endif
+#ifndef SPH_INTERACT_MINB_F64
+#define SPH_INTERACT_MINB_F64 4
+#endif
 #ifndef SPH_INTERACT_MINB_3D
-#define SPH_INTERACT_MINB_3D SPH_INTERACT_MINB
-#endif
-// the viscous pass and the update as two kernels (each with its own register budget) instead
-// of one (measured on the 1.2M cube: 0.73 ms against 0.86 for the fused kernel, the viscous
-// kernel at 8 blocks/SM, 7 and 6 being 3 % and 7 % slower; with the kernel factor in the
-// hand-over list 0.64 ms, 9 blocks/SM 0.70; on the 120k disk, with one viscous lane per
-// particle, 47 us against 39.5 us fused)
-#ifndef SPH_SPLIT_INTEGRATE_2D
-#define SPH_SPLIT_INTEGRATE_2D 0
-#endif
-#ifndef SPH_SPLIT_INTEGRATE_3D
-#define SPH_SPLIT_INTEGRATE_3D 1
+#define SPH_INTERACT_MINB_3D 6
 #endif
 #ifndef SPH_VISC_MINB_2D
-#define SPH_VISC_MINB_2D 8
+#define SPH_VISC_MINB_2D 12
 #endif
 #ifndef SPH_VISC_MINB_3D
-#define SPH_VISC_MINB_3D 8
+#define SPH_VISC_MINB_3D 10
 #endif
 #ifndef SPH_UPDATE_MINB
 #define SPH_UPDATE_MINB 6
-#endif
-#ifndef SPH_INTEGRATE_MINB_2D
-#define SPH_INTEGRATE_MINB_2D 7
-#endif
-#ifndef SPH_INTEGRATE_MINB_3D
-#define SPH_INTEGRATE_MINB_3D 6
 #endif
 // cells per support of the cell grid when the parameters leave the choice to the library
 // (measured with a 2.6h support: 2 in 2D are 9 % faster than 1; 1 in 3D is 45 % slower than 2)
@@ -218,11 +210,6 @@ static_assert(Lpp<2>::v % ILpp<2>::v == 0 && Lpp<3>::v % ILpp<3>::v == 0,
 #ifndef SPH_DEFAULT_CPS_3D
 #define SPH_DEFAULT_CPS_3D 2
 #endif
-// entries of the pressure-to-viscous hand-over list fetched together by the viscous pass
-#ifndef SPH_VISC_BATCH
-#define SPH_VISC_BATCH 2
-#endif
-
 // Whether a particle of intrinsic dimension di takes part in the step pass for dimension class
 // cls: 0 is the whole step at once; with Algorithm 1's feature loop in sequence (feature_order)
 // a step runs the passes cls = 1 .. D in turn and each moves the particles of its class, and an
@@ -238,6 +225,30 @@ template <typename T> __device__ __forceinline__ int inst_of(const State<T>& s, 
 }
 template <typename T> __device__ __forceinline__ bool live(const State<T>& s, int i, int k) {
     return k - __ldg(s.inst_off + i) < __ldg(s.inst_n + i);
+}
+
+// the sorted meta words of the batch's dimension (the same memory serves as scratch for plain
+// 32-bit metas while instances are re-packed)
+template <int D, typename T> __device__ __forceinline__ Meta<D>* meta_words(const State<T>& s) {
+    return reinterpret_cast<Meta<D>*>(s.Ms);
+}
+
+// meta (group and dimension) of sorted slot k
+template <typename T, int D> __device__ __forceinline__ unsigned slot_meta(const State<T>& s, int k) {
+    if constexpr (Rec<T, D>::packed) return MetaWord<D>::meta(__float_as_uint((float)s.P[k].w));
+    else return MetaWord<D>::meta(meta_words<D>(s)[k]);
+}
+
+// whether the list of slot k (n candidates) overflowed, and the place of its entry t
+template <typename T, int D> __device__ __forceinline__ bool list_overflowed(const State<T>& s, int k, int n) {
+    return n > ListShape<D>::ROW && (n > list_most<D>() || s.xcnt[k / CHUNK] > ListShape<D>::NXB);
+}
+template <typename T, int D>
+__device__ __forceinline__ size_t list_entry(const State<T>& s, int k, int t, unsigned long long xid) {
+    typedef ListShape<D> L;
+    if (t < L::ROW) return (size_t)k * L::ROW + t;
+    const int u = t - L::ROW, b = (int)(xid >> (8 * (u / L::XB))) & 255;
+    return s.xbase + (size_t)((k / CHUNK) * L::NXB + b) * L::XB + u % L::XB;
 }
 
 // the one-pass scan's tile states back to "nothing published" (grid-stride over any grid)
@@ -364,13 +375,19 @@ template <typename T, int D>
 void launch_store_state(const ConstSlotArrays<T>& s, const IoGrid& g, int ns, int n, double* x, int* group, double* v,
                         double* h, int* cnt, cudaStream_t st);
 
-// interact.cu
+// search.cu: the neighbour lists of the particles taking part in pass cls (in_pass; -1: of all);
+// tested (may be null) counts the candidate pairs tested
+template <typename T, int D>
+void launch_search(const State<T>& s, const One* one, cudaStream_t st, bool pdl = false, int cls = 0,
+                   unsigned long long* tested = nullptr);
+
+// interact.cu (over the lists of a search)
 template <typename T, int D>
 void launch_interact(const State<T>& s, const One* one, T* dbg_sigma, T* dbg_gamma, cudaStream_t st,
                      bool pdl = false, int cls = 0);
 template <typename T, int D>
 void launch_neighbors(const State<T>& s, int mode, int* counts, const long long* offsets, int* lists, cudaStream_t st);
-template <typename T, int D> void launch_pair_counts(const State<T>& s, unsigned long long* out2, cudaStream_t st);
+template <typename T, int D> void launch_pair_counts(const State<T>& s, unsigned long long* out, cudaStream_t st);
 
 // integrate.cu
 template <typename T, int D>
