@@ -18,6 +18,8 @@
 // A block serves BLOCK/LPP consecutive slots, which lie in one chunk and so in one instance:
 // the instance's grid and parameters are copied into shared memory once per block (a batch of
 // one passes them as kernel parameters instead).
+#include <type_traits>
+
 #include "walk.cuh"
 
 namespace sph {
@@ -243,11 +245,22 @@ __global__ void __launch_bounds__(BLOCK, (interact_minb<T, D>()))
     Pressure<T, D> c{s, g, p, dom};
     c.init(hi, mi, offi, li, ci);
     const bool over = active && list_overflowed<T, D>(s, k, n);
-    const bool uniform = sizeof(T) == 4 && __all_sync(FULL, !active || di == D);
     if constexpr (sizeof(T) == 4) {
-        if (uniform && active && !over) {
-            // all particles of the warp of full dimension, in single precision: packed arithmetic,
-            // two pairs per operation (for each pair the operations of Pressure::pair)
+        // single precision: packed arithmetic, two pairs per operation (for each pair the operations
+        // of Pressure::pair); compiled for warps whose particles are all of full dimension (most)
+        // and for mixed ones, whose powers and constants depend on the lane
+        auto sums_of = [&](auto full) {
+            constexpr bool FD = decltype(full)::value;
+            const int d = FD ? D : di;
+            // x1, x2 or x3 by the particle's dimension
+            auto pick = [&](f32x2 x1, f32x2 x2, f32x2 x3) -> f32x2 {
+                if (FD) return D == 2 ? x2 : x3;
+                const f32x2 low = d == 1 ? x1 : x2;
+                return D == 3 && d == 3 ? x3 : low;
+            };
+            const float A = d == 1 ? -20.0f * 1.5f
+                                   : d == 2 ? (float)(-20.0 * 7.0 / CUDART_PI) : (float)(-20.0 * 21.0 / (2.0 * CUDART_PI));
+            const f32x2 A2 = pack2(A, A);
             const f32x2 c02 = pack2(g.c0, g.c0), hi2 = pack2(hi, hi), hk2 = pack2(T(0.5) * kappa, T(0.5) * kappa), one2 = pack2(1.0f, 1.0f);
             const f32x2 nRi = pack2(-c.invRi, -c.invRi), hid2 = pack2(c.hi2d, c.hi2d);
             const unsigned long long xid = n > ListShape<D>::ROW ? s.xid[k] : 0ull;
@@ -292,7 +305,7 @@ __global__ void __launch_bounds__(BLOCK, (interact_minb<T, D>()))
                     const bool sa = ia && meta_group(ea) == gi, sb = ib && meta_group(eb) == gi;
                     const f32x2 r = pack2(root_of(r2a), root_of(r2b));
                     const f32x2 invR = pack2(fast_rcp(Ra), fast_rcp(Rb));
-                    const f32x2 h2 = mul2(h, h), hd = D == 2 ? h2 : mul2(h2, h);
+                    const f32x2 h2 = mul2(h, h), hd = pick(h, h2, mul2(h2, h));
                     const f32x2 S2 = add2(hid2, mul2(hd, hd));   // rho_i^-2 + rho_j^-2
                     // outside its support each kernel is zero, so the two sums need no predicate
                     f32x2 q = fma2(r, nRi, one2);
@@ -306,9 +319,7 @@ __global__ void __launch_bounds__(BLOCK, (interact_minb<T, D>()))
                     unpack2(q, xa, xb);
                     q = pack2(sa ? fmaxf(xa, 0.0f) : 0.0f, sb ? fmaxf(xb, 0.0f) : 0.0f);
                     const f32x2 i2 = mul2(invR, invR), i4 = mul2(i2, i2);
-                    const float A = D == 2 ? (float)(-20.0 * 7.0 / CUDART_PI) : (float)(-20.0 * 21.0 / (2.0 * CUDART_PI));
-                    const f32x2 kv =
-                        mul2(mul2(S2, mul2(D == 2 ? i4 : mul2(i4, invR), pack2(A, A))), mul2(mul2(q, q), q));
+                    const f32x2 kv = mul2(mul2(S2, mul2(pick(mul2(i2, invR), i4, mul2(i4, invR)), A2)), mul2(mul2(q, q), q));
                     F0 = fma2(kv, dx, F0);
                     F1 = fma2(kv, dy, F1);
                     if (D == 3) F2 = fma2(kv, dz, F2);
@@ -316,12 +327,12 @@ __global__ void __launch_bounds__(BLOCK, (interact_minb<T, D>()))
                     const bool na = r2a < qa, nb = r2b < qb;
                     fac[u] = na && r2a > 0.0f ? xa : 0.0f;
                     fac[u + 1] = nb && r2b > 0.0f ? xb : 0.0f;
-                    const bool wa = ia && na && meta_dim(ea) < D, wb = ib && nb && meta_dim(eb) < D;
+                    const bool wa = ia && na && meta_dim(ea) < d, wb = ib && nb && meta_dim(eb) < d;
                     if ((wa || wb) && p.boundary_corr != 0) {
                         float sx, sy;
                         unpack2(S2, sx, sy);
-                        if (wa) c.wall(D, root_of(r2a), Ra, sx, hj[u], ea, off[u], ma);
-                        if (wb) c.wall(D, root_of(r2b), Rb, sy, hj[u + 1], eb, off[u + 1], mb);
+                        if (wa) c.wall(d, root_of(r2a), Ra, sx, hj[u], ea, off[u], ma);
+                        if (wb) c.wall(d, root_of(r2b), Rb, sy, hj[u + 1], eb, off[u + 1], mb);
                     }
                 }
                 list_store(s.vr + e, fac);   // the pairs' kernel factors of Eq. 7
@@ -336,11 +347,15 @@ __global__ void __launch_bounds__(BLOCK, (interact_minb<T, D>()))
             if (D == 3) c.F[2] += fold(F2);
             c.sig += fold(S0);
             c.gam += fold(G0);
+        };
+        const bool full = __all_sync(FULL, !active || di == D);
+        if (active && !over) {
+            if (full) sums_of(std::true_type());
+            else sums_of(std::false_type());
         }
-    }
-    if (!uniform && active && !over) {   // pair by pair
+    } else if (active && !over) {   // pair by pair
         const unsigned long long xid = n > ListShape<D>::ROW ? s.xid[k] : 0ull;
-        constexpr int N = sizeof(T) == 4 ? U : 2;
+        constexpr int N = 2;
         for (int t = sub * N; t < n; t += LPP * N) {
             const size_t e = list_entry<T, D>(s, k, t, xid);
             int jj[N];
