@@ -147,14 +147,30 @@ template <typename T> __global__ void __launch_bounds__(SCAN1_THREADS) k_scan_on
     // occupancy words are rebuilt by the gather
     for (int t = tile * SCAN1_THREADS + threadIdx.x; t < s.nocc * OCCW; t += gridDim.x * SCAN1_THREADS) s.occ[t] = 0u;
     const int base = tile * SCAN1_TILE + threadIdx.x * SCAN1_ITEMS;
+    static_assert(SCAN1_ITEMS % 4 == 0, "cells are read and written four at a time");
+    const bool whole = base + SCAN1_ITEMS <= ncell;
     int loc[SCAN1_ITEMS];
     int v = 0;
+    if (whole) {
+        const int4* const cn = reinterpret_cast<const int4*>(s.count + base);
+        const int4* const cs = reinterpret_cast<const int4*>(s.cell_start + base);
+        int old[SCAN1_ITEMS + 1];
+        old[SCAN1_ITEMS] = s.cell_start[base + SCAN1_ITEMS];
 #pragma unroll
-    for (int k = 0; k < SCAN1_ITEMS; ++k) {
-        loc[k] = 0;
-        if (base + k < ncell) loc[k] = s.count[base + k] - s.cell_start[base + k + 1];
-        v += loc[k];
+        for (int k = 0; k < SCAN1_ITEMS / 4; ++k) {
+            const int4 c = cn[k], o = cs[k];
+            loc[4 * k] = c.x, loc[4 * k + 1] = c.y, loc[4 * k + 2] = c.z, loc[4 * k + 3] = c.w;
+            old[4 * k] = o.x, old[4 * k + 1] = o.y, old[4 * k + 2] = o.z, old[4 * k + 3] = o.w;
+        }
+#pragma unroll
+        for (int k = 0; k < SCAN1_ITEMS; ++k) loc[k] -= old[k + 1];
+    } else {
+#pragma unroll
+        for (int k = 0; k < SCAN1_ITEMS; ++k)
+            loc[k] = base + k < ncell ? s.count[base + k] - s.cell_start[base + k + 1] : 0;
     }
+#pragma unroll
+    for (int k = 0; k < SCAN1_ITEMS; ++k) v += loc[k];
     int agg;
     int ex = block_exclusive_scan(v, ws, agg);
     if (threadIdx.x < 32) {   // warp 0: publish, then look back 32 tiles at a time
@@ -200,12 +216,25 @@ template <typename T> __global__ void __launch_bounds__(SCAN1_THREADS) k_scan_on
     __syncthreads();
     ex += sh_prefix;
 #pragma unroll
-    for (int k = 0; k < SCAN1_ITEMS; ++k) {
-        if (base + k < ncell) {
-            s.cell_start[base + k] = ex;
-            s.count[base + k] = ex;    // scatter cursor
+    for (int k = 0; k < SCAN1_ITEMS; ++k) {   // loc: the start of the cell, also its scatter cursor
+        const int n = loc[k];
+        loc[k] = ex;
+        ex += n;
+    }
+    if (whole) {
+#pragma unroll
+        for (int k = 0; k < SCAN1_ITEMS / 4; ++k) {
+            const int4 e = make_int4(loc[4 * k], loc[4 * k + 1], loc[4 * k + 2], loc[4 * k + 3]);
+            reinterpret_cast<int4*>(s.cell_start + base)[k] = e;
+            reinterpret_cast<int4*>(s.count + base)[k] = e;
         }
-        ex += loc[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < SCAN1_ITEMS; ++k)
+            if (base + k < ncell) {
+                s.cell_start[base + k] = loc[k];
+                s.count[base + k] = loc[k];
+            }
     }
     if (base + SCAN1_ITEMS >= ncell && base < ncell) s.cell_start[ncell] = ex;   // the thread holding the last cell
 }

@@ -276,12 +276,13 @@ __device__ __forceinline__ void own_cell(const Grid& g, const State<T>& s, int k
 constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_ITEMS = 4;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
-// cells per thread and threads per tile of the step's one-pass scan (measured: 2 is 6 % faster
-// than 4 in the rebuild, 8 and 16 are 27 % and 86 % slower; again with the 2.6h support and its
-// 1.41M-cell 2D grid: 1 / 4 / 8 per thread 20 / 9 / 65 % slower than 2; 512 x 2 and 256 x 4
-// threads x cells equal to 1024 x 2 within 1 %, 512 x 4 and 256 x 8 9 % and 35 % slower)
+// cells per thread (read and written as 16-byte words) and threads per tile of the step's one-pass
+// scan (bound by DRAM and the tiles' chain: 200 MB in 45 us on the 12M cells of the 83k graded cube;
+// measured, rebuild in us, 2 cells per thread word by word / 4 / 8 / 8 with 512 threads: 20k disk
+// 16.5 / 16.2 / 17.6 / 16.3, 1M disk 111 / 84.6 / 83.7 / 82.9, 83k cube 105 / 73.2 / 72.3 / 72.4, 1.2M
+// cube 106 / 90.0 / 91.2 / 90.3)
 #ifndef SPH_SCAN1_ITEMS
-#define SPH_SCAN1_ITEMS 2
+#define SPH_SCAN1_ITEMS 4
 #endif
 #ifndef SPH_SCAN1_THREADS
 #define SPH_SCAN1_THREADS 1024
