@@ -327,14 +327,21 @@ def sph_mesh_run_until_converged(m, max_iters):
     return st == SPH_OK, it.value
 
 
+def _filled(got, **arrays):
+    """Arrays of which the library has written the first `got` elements, zero beyond them."""
+    for a in arrays.values():
+        a[got:] = 0
+    return arrays
+
+
 def sph_mesh_positions(m, n):
-    x = np.zeros((n, 3))
-    g = np.zeros(n, np.int32)
-    v = np.zeros((n, 3))
-    h = np.zeros(n)
+    x = np.empty((n, 3))
+    g = np.empty(n, np.int32)
+    v = np.empty((n, 3))
+    h = np.empty(n)
     got = C.c_int64(0)
     _check(lib().sph_mesh_positions(m, _p(x), _p(g), _p(v), _p(h), n, C.addressof(got)))
-    return dict(x=x, group=g, v=v, h=h)
+    return _filled(got.value, x=x, group=g, v=v, h=h)
 
 
 def sph_mesh_report(m) -> sph_report:
@@ -458,13 +465,13 @@ def sph_batch_run_until_converged(b, max_iters):
 
 
 def sph_batch_positions(b, inst, n):
-    x = np.zeros((n, 3))
-    g = np.zeros(n, np.int32)
-    v = np.zeros((n, 3))
-    h = np.zeros(n)
+    x = np.empty((n, 3))
+    g = np.empty(n, np.int32)
+    v = np.empty((n, 3))
+    h = np.empty(n)
     got = C.c_int64(0)
     _check(lib().sph_batch_positions(b, int(inst), _p(x), _p(g), _p(v), _p(h), n, C.addressof(got)))
-    return dict(x=x, group=g, v=v, h=h)
+    return _filled(got.value, x=x, group=g, v=v, h=h)
 
 
 def sph_batch_reports(b, n_inst):
