@@ -545,6 +545,7 @@ __global__ void __launch_bounds__(BLOCK) k_predict(State<T> s, One one, const Ct
 // 2 a b / (a + b) for a, b >= 0 (0 where the sum is 0)
 template <typename T> __device__ __forceinline__ T harmonic(T a, T b) {
     const T s = a + b;
+    if (sizeof(T) == 8 && s > T(1e-280)) return T(2) * a * b * fast_rcp(s);   // s far from the range's end
     return s > T(0) ? T(2) * a * b / s : T(0);
 }
 

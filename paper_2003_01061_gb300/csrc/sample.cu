@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(SB) k_feature_integral(const Domain* dmp, cons
             }
             if (inside(dm, x, xf, size)) {
                 const double h = quad_h(z, x, xf, size);
-                acc += cell / (D == 3 ? h * h * h : h * h);
+                acc += cell * fast_rcp(D == 3 ? h * h * h : h * h);
             }
         } else if (KIND == SPH_FEAT_SEGMENT) {
             const double t = (i + 0.5) * inq;
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(SB) k_feature_integral(const Domain* dmp, cons
             const double si = (((int)i & last) + 0.5) * inq * f.g[9], tj = ((int)(i >> ln) + 0.5) * inq * f.g[10];
             for (int a = 0; a < 3; ++a) x[a] = f.g[a] + si * f.g[3 + a] + tj * f.g[6 + a];
             const double h = samp_h(z, x);
-            acc += cell / (h * h);
+            acc += cell * fast_rcp(h * h);
         } else if (KIND == SPH_FEAT_SPHERE) {
             const int ii = (int)(i >> (ln + 1)), jj = (int)i & (2 * nq - 1);
             const double th = CUDART_PI * (ii + 0.5) * inq, ph = CUDART_PI * (jj + 0.5) * inq;
