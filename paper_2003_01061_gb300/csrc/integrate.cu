@@ -804,7 +804,7 @@ __global__ void __launch_bounds__(BLOCK, (FUSED || sizeof(T) == 8 ? 4 : (D == 2 
 }
 
 template <typename T, int D, bool ONE>
-__global__ void __launch_bounds__(BLOCK, (sizeof(T) == 4 ? SPH_UPDATE_MINB : 4))
+__global__ void __launch_bounds__(BLOCK, (sizeof(T) == 4 ? (D == 2 ? SPH_UPDATE_MINB_2D : SPH_UPDATE_MINB_3D) : 4))
     k_update(State<T> s, One one, const Ctrl* use, Out<T> o, int cls) {
     dep_launch();
     dep_wait();

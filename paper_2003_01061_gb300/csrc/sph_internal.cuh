@@ -183,7 +183,8 @@ static_assert(CHUNK % (BLOCK / Lpp<2>::v) == 0 && CHUNK % (BLOCK / Lpp<3>::v) ==
 // per thread, trading spills for warps in flight (measured, search and pressure pass in us: 2D, 1M
 // disk, 5 / 6 / 7 / 8 blocks 499 / 472 / 443 / 428; 3D, 1.2M cube, 5 / 6 / 7 / 8 blocks 1541 / 1499 /
 // 1504 / 1595; FP64, 40k cube, 4 / 6 blocks 791 / 990; viscous sum and update: 1M disk 6 / 8 / 10 /
-// 12 blocks 219 / 201 / 182 / 172, 1.2M cube 8 / 10 / 12 blocks 392 / 362 / 439)
+// 12 blocks 219 / 201 / 182 / 172, 1.2M cube 8 / 10 / 12 blocks 392 / 362 / 439; update alone at 6 /
+// 8 blocks: the same stage 171.5 / 167.5 us on the 1M disk, 56.0 / 59.3 on the 83k cube)
 #ifndef SPH_INTERACT_MINB
 #define SPH_INTERACT_MINB 8
 #endif
@@ -199,8 +200,11 @@ static_assert(CHUNK % (BLOCK / Lpp<2>::v) == 0 && CHUNK % (BLOCK / Lpp<3>::v) ==
 #ifndef SPH_VISC_MINB_3D
 #define SPH_VISC_MINB_3D 10
 #endif
-#ifndef SPH_UPDATE_MINB
-#define SPH_UPDATE_MINB 6
+#ifndef SPH_UPDATE_MINB_2D
+#define SPH_UPDATE_MINB_2D 8
+#endif
+#ifndef SPH_UPDATE_MINB_3D
+#define SPH_UPDATE_MINB_3D 6
 #endif
 // cells per support of the cell grid when the parameters leave the choice to the library
 // (measured with a 2.6h support: 2 in 2D are 9 % faster than 1; 1 in 3D is 45 % slower than 2)

@@ -107,12 +107,14 @@ __device__ __forceinline__ void list_store(float* p, const float (&f)[2]) {
 }
 
 // ---- the search of one warp ----
-#ifndef SPH_SEG_SPAN
-#define SPH_SEG_SPAN 6
-#endif
-// Longest segment, in cells of its row: a longer one has a wider bounding box, a shorter one
-// splits more warps.
-constexpr int SEG_SPAN = SPH_SEG_SPAN;
+// Longest segment, in cells of its row, of a warp that searches for cl particles: a longer one has a
+// wider bounding box, a shorter one splits more warps.  Measured, whole step in us: 3D, cl = 2 with 1 /
+// 2 / 3 / 6, 26k ball in three passes 280 / 280 / 315 / 351; cl = 8 with 3 / 4 / 5 / 6, batch of 340k 724 /
+// 728 / 732 / 744; cl = 16 with 4 / 6 / 10, 1.2M cube 1941 / 1925 / 1953; 2D, cl = 8 with 6 / 8 / 10 / 14,
+// 120k disk 136.2 / 133.9 / 133.4 / 135.4; cl = 16 with 6 / 12 / 16 / 24, 1M disk 668 / 658 / 655 / 656.
+constexpr int seg_span(int D, int cl) {
+    return D == 2 ? (cl <= 4 ? 6 : cl == 8 ? 10 : 16) : (cl <= 4 ? 2 : cl == 8 ? 3 : 6);
+}
 
 template <int CL> struct alignas(16) SearchWarp {
     float4 me[CL];                   // pairs of particles: (-x, -x', -y, -y'), (-z, -z', a, a')
@@ -184,11 +186,13 @@ __device__ __forceinline__ void stg_if_less(float a, float b, char* p, int j) {
 // shared memory, two particles per packed operation).  The hits of a particle are appended, in
 // candidate order, to its row of the neighbour lists.
 //
-// What bounds it: the instruction stream, about 5.7k warp instructions per 8 particles on a 300k
-// cube (issue slots 67 % busy), a third of it in the ~27 groups of candidates, a quarter in the
-// ~10 groups tested, the rest in segments and rows.  The walk it replaces, 8 lanes searching for
+// What bounds it: the instruction stream, about 6k warp instructions per 8 particles on a 300k cube
+// (issue slots 73 % busy), a third of it in the ~27 groups of candidates, a third in the ~10 groups
+// tested, the rest in segments and rows; on small states the slowest warp's chain of loads.
+// Loading the next candidates ahead of the tests gained nothing at 32 warps per SM (605 us per step
+// with, 597 without, on that cube).  The walk it replaces, 8 lanes searching for
 // their own particle and working off its pairs as they came, took 2.9k per particle for search and
-// pair sums together (pressure pass of the 1.2M cube 3.6 ms; search and pressure pass now 1.5 ms).
+// pair sums together (pressure pass of the 1.2M cube 3.6 ms; search and pressure pass now 1.47 ms).
 // Measured on the way: testing every candidate against all particles without the box test 211 M
 // instead of 172 M instructions on that cube; pair sums inside the search kernel, from pools in
 // shared memory, 80 registers with spills in both and 1.8 ms.
@@ -264,7 +268,7 @@ __device__ __forceinline__ int warp_search(const Grid& g, const State<T>& s, Sea
         int sc[3] = {0, 0, 0};
         for (int a = 0; a < D; ++a) sc[a] = __shfl_sync(FULL, ci[a], ll);
         const bool in = active && ((pend >> (lane - sub)) & 1u) && li == sl && ci[1] == sc[1] &&
-                        (D == 2 || ci[2] == sc[2]) && (unsigned)(ci[0] - sc[0]) <= (unsigned)SEG_SPAN;
+                        (D == 2 || ci[2] == sc[2]) && (unsigned)(ci[0] - sc[0]) <= (unsigned)seg_span(D, CL);
         const unsigned seg = __ballot_sync(FULL, in && sub == 0);
         pend &= ~seg;
         const float x[3] = {fi.x, fi.y, fi.z};
@@ -406,26 +410,19 @@ __device__ __forceinline__ int warp_search(const Grid& g, const State<T>& s, Sea
             __syncwarp();
             tested += (unsigned long long)total * (unsigned)__popc(seg);
             const bool last = r0 + 32 >= nrows;
-            // this lane's candidate among those from c on, loaded one group ahead of its test
-            int c = 0, started = 0, jn = 0;
-            float4 fn = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            auto fetch = [&]() {
-                const unsigned at = (unsigned)(excl - c);   // rows that start here
-                const unsigned heads = __reduce_or_sync(FULL, len > 0 && at < 32u ? 1u << at : 0u);
-                const int ord = started + __popc(heads & (lt | (1u << lane))) - 1;
-                started += __popc(heads);
-                jn = min(c + lane, total - 1) + lds_i(sh_me + DELTA + 4 * ord);   // past the end: the last again
-                fn = s.F[jn];
-            };
-            if (total > 0) fetch();
+            int c = 0, started = 0;
             do {
                 if (c < total) {
                     // ---- 32 candidates, one per lane: those near the box into the ring ----
-                    const float4 f = fn;
-                    const int j = jn;
+                    const unsigned first_at = (unsigned)(excl - c);   // rows that start here
+                    const unsigned heads = __reduce_or_sync(FULL, len > 0 && first_at < 32u ? 1u << first_at : 0u);
+                    const int ord = started + __popc(heads & (lt | (1u << lane))) - 1;
+                    started += __popc(heads);
+                    // past the end: the last candidate again
+                    const int j = min(c + lane, total - 1) + lds_i(sh_me + DELTA + 4 * ord);
+                    const float4 f = s.F[j];
                     const bool there = c + lane < total;
                     c += 32;
-                    if (c < total) fetch();
                     const float dx = fmaxf(fmaxf(b0[0] - f.x, f.x - b1[0]), 0.0f);
                     const float dy = fmaxf(fmaxf(b0[1] - f.y, f.y - b1[1]), 0.0f);
                     float d2 = fmaf(dy, dy, dx * dx);
