@@ -157,36 +157,43 @@ __device__ bool accept(const Domain& dm, const Sizing& z, const Feat& f, const d
     }
 }
 
+// One pass over candidates of several features: blocks block0[q] .. block0[q + 1] take the next
+// candidates, from c0[q] on, of feature k[q], which wants its first want[q] accepted ones at
+// out0[q] (particles).
+struct SamplePass {
+    int n;
+    int k[MAXF];
+    int block0[MAXF + 1];
+    long long c0[MAXF], want[MAXF], out0[MAXF];
+};
+__device__ __forceinline__ int pass_entry(const SamplePass& ps) {
+    int q = 0;
+    while (q + 1 < ps.n && (int)blockIdx.x >= ps.block0[q + 1]) ++q;
+    return q;
+}
+
 // pass 1: accepted candidates per block
-__global__ void __launch_bounds__(SB) k_sample_count(const Domain* dmp, const Sizing* zp, int k,
-                                                     unsigned long long seed, long long c0, long long nc,
-                                                     int* block_count) {
+__global__ void __launch_bounds__(SB) k_sample_count(const Domain* dmp, const Sizing* zp, unsigned long long seed,
+                                                     const __grid_constant__ SamplePass ps, int* block_count) {
     const Domain& dm = *dmp;
-    const long long c = c0 + (long long)blockIdx.x * SB + threadIdx.x;
-    bool ok = false;
-    if (c < c0 + nc) {
-        double u[4], x[3];
-        uniforms(seed, k, c, u);
-        ok = accept(dm, *zp, dm.f[k], u, x);
-    }
-    const int n = __syncthreads_count(ok ? 1 : 0);
+    const int q = pass_entry(ps), k = ps.k[q];
+    double u[4], x[3];
+    uniforms(seed, k, ps.c0[q] + (long long)(blockIdx.x - ps.block0[q]) * SB + threadIdx.x, u);
+    const int n = __syncthreads_count(accept(dm, *zp, dm.f[k], u, x) ? 1 : 0);
     if (threadIdx.x == 0) block_count[blockIdx.x] = n;
 }
 
-// pass 2: accepted candidates written in candidate order, the first `want` of them
-__global__ void __launch_bounds__(SB) k_sample_emit(const Domain* dmp, const Sizing* zp, int k,
-                                                    unsigned long long seed, long long c0, long long nc,
-                                                    const long long* block_off, long long want, double* out) {
+// pass 2: accepted candidates written in candidate order, the first `want` of them (block_off: the
+// accepted candidates of the block's feature before it)
+__global__ void __launch_bounds__(SB) k_sample_emit(const Domain* dmp, const Sizing* zp, unsigned long long seed,
+                                                    const __grid_constant__ SamplePass ps, const long long* block_off,
+                                                    double* out) {
     __shared__ int wsum[SB / 32];
     const Domain& dm = *dmp;
-    const long long c = c0 + (long long)blockIdx.x * SB + threadIdx.x;
-    bool ok = false;
-    double x[3] = {0.0, 0.0, 0.0};
-    if (c < c0 + nc) {
-        double u[4];
-        uniforms(seed, k, c, u);
-        ok = accept(dm, *zp, dm.f[k], u, x);
-    }
+    const int q = pass_entry(ps), k = ps.k[q];
+    double u[4], x[3] = {0.0, 0.0, 0.0};
+    uniforms(seed, k, ps.c0[q] + (long long)(blockIdx.x - ps.block0[q]) * SB + threadIdx.x, u);
+    const bool ok = accept(dm, *zp, dm.f[k], u, x);
     const unsigned bal = __ballot_sync(0xffffffffu, ok);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (lane == 0) wsum[wid] = __popc(bal);
@@ -194,8 +201,8 @@ __global__ void __launch_bounds__(SB) k_sample_emit(const Domain* dmp, const Siz
     int before = 0;
     for (int w = 0; w < wid; ++w) before += wsum[w];
     const long long rank = block_off[blockIdx.x] + before + __popc(bal & ((1u << lane) - 1u));
-    if (ok && rank < want)
-        for (int a = 0; a < 3; ++a) out[3 * rank + a] = x[a];
+    if (ok && rank < ps.want[q])
+        for (int a = 0; a < 3; ++a) out[3 * (ps.out0[q] + rank) + a] = x[a];
 }
 
 // phi(x) > 0 as samp_phi has it.  Single precision decides wherever the level set is clearly off
@@ -448,56 +455,86 @@ double acceptance_estimate(const Domain& dm, const Sizing& z, int k, long long n
 
 cudaError_t sample_features(const Domain& dm, const Sizing& z, const Domain* d_dom, const Sizing* d_siz,
                             unsigned long long seed, const int64_t* counts, cudaStream_t st, double* d_out) {
-    // candidates per pass: enough for the remaining count at the expected acceptance, so that
-    // one pass (one host round trip) usually suffices; a short pass is followed by another one
-    // sized by the acceptance seen so far.  The result does not depend on the pass sizes: it is
-    // always the first accepted candidates in candidate order.
-    constexpr long long MAXB = 1LL << 26;
+    // Candidates per pass: enough for the remaining count at the expected acceptance, so that one
+    // pass usually suffices; a short one is followed by another sized by the acceptance seen so
+    // far.  All features share the passes (two kernels and one host round trip each, where one pass
+    // per feature took 28 round trips for a cube: 1.2 ms).  The result does not depend on the pass
+    // sizes: it is always the first accepted candidates in candidate order.
+    constexpr long long MAXB = 1LL << 26;   // candidates per pass
+    struct Feature {
+        long long got = 0, c0 = 0, seen = 0, taken = 0;
+        double p = 1.0;
+    };
+    std::vector<Feature> fs(dm.nf);
+    std::vector<long long> base(dm.nf + 1, 0);
+    for (int k = 0; k < dm.nf; ++k) {
+        base[k + 1] = base[k] + counts[k];
+        if (counts[k] > 0) fs[k].p = acceptance_estimate(dm, z, k, counts[k]);
+    }
     int* d_cnt = nullptr;
     long long* d_off = nullptr;
-    cudaError_t e = cudaMallocAsync(&d_cnt, sizeof(int) * (MAXB / SB), st);
-    if (e == cudaSuccess) e = cudaMallocAsync(&d_off, sizeof(long long) * (MAXB / SB), st);
-    std::vector<int> cnt(MAXB / SB);
-    std::vector<long long> off(MAXB / SB);
-    long long base = 0;
-    for (int k = 0; k < dm.nf && e == cudaSuccess; ++k) {
-        const long long want = counts[k];
-        if (want > 0 && dm.f[k].kind == SPH_FEAT_POINT) {   // the point itself
-            double x[3] = {0.0, 0.0, 0.0};
-            for (int a = 0; a < dm.D; ++a) x[a] = dm.f[k].g[a];
-            e = cudaMemcpyAsync(d_out + 3 * base, x, sizeof x, cudaMemcpyHostToDevice, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            base += want;
-            continue;
-        }
-        double p = acceptance_estimate(dm, z, k, want);
-        long long got = 0, c0 = 0, seen = 0, taken = 0;
-        while (got < want && e == cudaSuccess) {
-            const double need = (double)(want - got) / p;
+    size_t cap = 0;   // blocks d_cnt and d_off hold
+    std::vector<int> cnt;
+    std::vector<long long> off;
+    cudaError_t e = cudaSuccess;
+    while (e == cudaSuccess) {
+        SamplePass ps;
+        ps.n = 0;
+        ps.block0[0] = 0;
+        long long room = MAXB;
+        for (int k = 0; k < dm.nf; ++k) {
+            Feature& f = fs[k];
+            if (f.got >= counts[k] || room == 0) continue;
+            const double need = (double)(counts[k] - f.got) / f.p;
             long long nc = (long long)(1.05 * need + 6.0 * std::sqrt(need)) + 4096;
-            nc = std::min(MAXB, (nc + SB - 1) / SB * SB);
-            const int nblk = (int)(nc / SB);
-            k_sample_count<<<nblk, SB, 0, st>>>(d_dom, d_siz, k, seed, c0, nc, d_cnt);
-            e = cudaMemcpyAsync(cnt.data(), d_cnt, sizeof(int) * nblk, cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            if (dm.f[k].kind == SPH_FEAT_POINT) nc = counts[k];   // every candidate is the point itself
+            nc = std::min(room, (nc + SB - 1) / SB * SB);
+            ps.k[ps.n] = k;
+            ps.c0[ps.n] = f.c0;
+            ps.want[ps.n] = counts[k];
+            ps.out0[ps.n] = base[k];
+            ps.block0[ps.n + 1] = ps.block0[ps.n] + (int)(nc / SB);
+            room -= nc;
+            ps.n += 1;
+        }
+        if (ps.n == 0) break;
+        const int nblk = ps.block0[ps.n];
+        if ((size_t)nblk > cap) {
+            if (d_cnt) cudaFreeAsync(d_cnt, st);
+            if (d_off) cudaFreeAsync(d_off, st);
+            d_cnt = nullptr;
+            d_off = nullptr;
+            cap = (size_t)nblk;
+            e = cudaMallocAsync(&d_cnt, sizeof(int) * cap, st);
+            if (e == cudaSuccess) e = cudaMallocAsync(&d_off, sizeof(long long) * cap, st);
             if (e != cudaSuccess) break;
-            long long run = got;
-            for (int b = 0; b < nblk; ++b) {
+            cnt.resize(cap);
+            off.resize(cap);
+        }
+        k_sample_count<<<nblk, SB, 0, st>>>(d_dom, d_siz, seed, ps, d_cnt);
+        e = cudaMemcpyAsync(cnt.data(), d_cnt, sizeof(int) * nblk, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) break;
+        for (int q = 0; q < ps.n; ++q) {
+            Feature& f = fs[ps.k[q]];
+            long long run = f.got;
+            for (int b = ps.block0[q]; b < ps.block0[q + 1]; ++b) {
                 off[b] = run;
                 run += cnt[b];
             }
-            e = cudaMemcpyAsync(d_off, off.data(), sizeof(long long) * nblk, cudaMemcpyHostToDevice, st);
-            if (e != cudaSuccess) break;
-            k_sample_emit<<<nblk, SB, 0, st>>>(d_dom, d_siz, k, seed, c0, nc, d_off, want, d_out + 3 * base);
-            e = cudaStreamSynchronize(st);   // off is reused by the next pass
-            seen += nc;
-            taken += run - got;
-            got = std::min(run, want);
-            c0 += nc;
-            p = std::max(1e-9, (double)std::max<long long>(taken, 1) / (double)seen);
-            if (got < want && c0 >= (1LL << 36)) e = cudaErrorInvalidValue;   // acceptance too small
+            const long long nc = (long long)(ps.block0[q + 1] - ps.block0[q]) * SB;
+            f.seen += nc;
+            f.taken += run - f.got;
+            f.got = std::min<long long>(run, counts[ps.k[q]]);
+            f.c0 += nc;
+            f.p = std::max(1e-9, (double)std::max<long long>(f.taken, 1) / (double)f.seen);
+            if (f.got < counts[ps.k[q]] && f.c0 >= (1LL << 36)) e = cudaErrorInvalidValue;   // acceptance too small
         }
-        base += want;
+        if (e != cudaSuccess) break;
+        e = cudaMemcpyAsync(d_off, off.data(), sizeof(long long) * nblk, cudaMemcpyHostToDevice, st);
+        if (e != cudaSuccess) break;
+        k_sample_emit<<<nblk, SB, 0, st>>>(d_dom, d_siz, seed, ps, d_off, d_out);
+        e = cudaStreamSynchronize(st);   // off is reused by the next pass
     }
     if (d_cnt) cudaFreeAsync(d_cnt, st);
     if (d_off) cudaFreeAsync(d_off, st);
