@@ -722,7 +722,7 @@ __device__ __forceinline__ void update_one(const State<T>& s, const Grid& g, con
 
 
 template <typename T, int D, bool ONE, bool FUSED>
-__global__ void __launch_bounds__(BLOCK, (FUSED || sizeof(T) == 8 ? 4 : (D == 2 ? SPH_VISC_MINB_2D : SPH_VISC_MINB_3D)))
+__global__ void __launch_bounds__(BLOCK, (FUSED ? SPH_FUSED_MINB : sizeof(T) == 8 ? 4 : (D == 2 ? SPH_VISC_MINB_2D : SPH_VISC_MINB_3D)))
     k_visc(const __grid_constant__ State<T> s, const __grid_constant__ One one, const Ctrl* use, Out<T> o, int cls) {
     dep_launch();
     dep_wait();

@@ -226,10 +226,31 @@ __device__ __forceinline__ bool inside(const Domain& dm, const double x[3], cons
     return samp_phi(dm, x) > 0.0;
 }
 
-// h_t(x) as samp_h has it, without the FP64 roots of reference circles and spheres that single
+// sqrt(s) of a normal s: the hardware's estimate of 1/sqrt and one third-order step of Newton's
+// iteration (e = 1 - s y^2, sqrt = s y (1 + e/2 + 3/8 e^2)), within an ulp; the acceptance test of
+// the sampling keeps the correctly rounded root
+__device__ __forceinline__ double quad_root(double s) {
+    if (!(s > 1e-280 && s < 1e280)) return sqrt(s);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
+    const double t = s * y, e = fma(-t, y, 1.0);
+    return fma(t * e, fma(0.375, e, 0.5), t);
+}
+
+// h_t(x) as samp_h has it but for the rounding of the root, and without the FP64 roots of reference circles and spheres that single
 // precision shows to be clearly farther than the nearest one.
 __device__ __forceinline__ double quad_h(const Sizing& z, const double x[3], const float xf[3], float size) {
-    if (z.kind != 1 || z.nref < 2) return samp_h(z, x);
+    auto root_dist = [&](const double* c) {
+        const double d0 = x[0] - c[0], d1 = x[1] - c[1], d2 = x[2] - c[2];
+        return quad_root(fma(d2, d2, fma(d1, d1, d0 * d0)));
+    };
+    auto clamp = [&](double h) {
+        if (h < z.lo) h = z.lo;
+        return h > z.hi ? z.hi : h;
+    };
+    if (z.kind == 2) return clamp(z.a + z.b * root_dist(z.q));
+    if (z.kind != 1 || z.nref < 1) return samp_h(z, x);
+    if (z.nref == 1) return clamp(z.a + z.b * fabs(root_dist(z.rc[0]) - z.rr[0]));
     float best = 3e38f, next = 3e38f;
     int kb = 0;
     for (int k = 0; k < z.nref; ++k) {
@@ -245,25 +266,18 @@ __device__ __forceinline__ double quad_h(const Sizing& z, const double x[3], con
         }
     }
     if (!(next - best > size * 0x1p-16f)) return samp_h(z, x);
-    double h = dadd(z.a, dmul(z.b, fabs(dsub(dist_n(x, z.rc[kb], 3), z.rr[kb]))));
-    if (h < z.lo) h = z.lo;
-    if (h > z.hi) h = z.hi;
-    return h;
+    return clamp(z.a + z.b * fabs(root_dist(z.rc[kb]) - z.rr[kb]));
 }
 
 // Midpoint-rule integral of rho_t over feature k (Eqs. 10, 11), per-block partial sums.  The
 // quadrature sizes are powers of two (nq = 2^ln), so the divisions by nq are exact and a point's
 // indices are bits of its number; what does not depend on the point is computed before the loop.
-// Bound by the FP64 pipe, two multiply-adds per SM and clock: a volume point now costs one root and
-// one quotient (about 50 FP64 instructions), where three quotients for the cell size and a second
-// root for the level set made it about 130 (256^3 points, one hole: 4.2 ms before).
+// Bound by the FP64 pipe, two multiply-adds per SM and clock: a volume point costs one root and one
+// reciprocal (about 30 FP64 instructions), where three quotients for the cell size and a second
+// root for the level set made it about 130.
 template <int KIND>
-__global__ void __launch_bounds__(SB) k_feature_integral(const Domain* dmp, const Sizing* zp, int k, long long npts,
-                                                         int ln, double* partial) {
-    __shared__ double ws[SB / 32];
-    const Domain& dm = *dmp;
-    const Sizing& z = *zp;
-    const Feat& f = dm.f[k];
+__device__ __forceinline__ double integral_share(const Domain& dm, const Sizing& z, const Feat& f, long long npts, int ln,
+                                                 int block, int nblocks) {
     const int D = dm.D, nq = 1 << ln, last = nq - 1;
     const double inq = 1.0 / nq;
     float size = 0.0f;   // of the domain, with its distance from the origin
@@ -291,7 +305,7 @@ __global__ void __launch_bounds__(SB) k_feature_integral(const Domain* dmp, cons
     if (KIND == SPH_FEAT_CIRCLE) cell = 2.0 * CUDART_PI * f.g[2] * inq;
     if (KIND == SPH_FEAT_RECT) cell = (f.g[9] * inq) * (f.g[10] * inq);
     double acc = 0.0;
-    for (long long i = (long long)blockIdx.x * SB + threadIdx.x; i < npts; i += (long long)gridDim.x * SB) {
+    for (long long i = (long long)block * SB + threadIdx.x; i < npts; i += (long long)nblocks * SB) {
         double x[3] = {0.0, 0.0, 0.0};
         if (KIND == SPH_FEAT_VOLUME) {
             float xf[3];
@@ -306,16 +320,19 @@ __global__ void __launch_bounds__(SB) k_feature_integral(const Domain* dmp, cons
         } else if (KIND == SPH_FEAT_SEGMENT) {
             const double t = (i + 0.5) * inq;
             for (int a = 0; a < 3; ++a) x[a] = f.g[a] + t * dx[a];
-            acc += cell / samp_h(z, x);
+            const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
+            acc += cell / quad_h(z, x, xf, size);
         } else if (KIND == SPH_FEAT_CIRCLE) {
             const double th = 2.0 * CUDART_PI * (i + 0.5) * inq;
             x[0] = f.g[0] + f.g[2] * cos(th);
             x[1] = f.g[1] + f.g[2] * sin(th);
-            acc += cell / samp_h(z, x);
+            const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
+            acc += cell / quad_h(z, x, xf, size);
         } else if (KIND == SPH_FEAT_RECT) {
             const double si = (((int)i & last) + 0.5) * inq * f.g[9], tj = ((int)(i >> ln) + 0.5) * inq * f.g[10];
             for (int a = 0; a < 3; ++a) x[a] = f.g[a] + si * f.g[3 + a] + tj * f.g[6 + a];
-            const double h = samp_h(z, x);
+            const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
+            const double h = quad_h(z, x, xf, size);
             acc += cell * fast_rcp(h * h);
         } else if (KIND == SPH_FEAT_SPHERE) {
             const int ii = (int)(i >> (ln + 1)), jj = (int)i & (2 * nq - 1);
@@ -327,9 +344,36 @@ __global__ void __launch_bounds__(SB) k_feature_integral(const Domain* dmp, cons
             x[0] = f.g[0] + R * st * cp;
             x[1] = f.g[1] + R * st * sp;
             x[2] = f.g[2] + R * ct;
-            const double h = samp_h(z, x);
+            const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
+            const double h = quad_h(z, x, xf, size);
             acc += R * R * st * (CUDART_PI * inq) * (CUDART_PI * inq) / (h * h);
         }
+    }
+    return acc;
+}
+
+// all features in one launch: blocks block0[q] .. block0[q + 1] share the points of feature k[q]
+struct IntegralPass {
+    int n;
+    int k[MAXF], ln[MAXF], block0[MAXF + 1];
+    long long npts[MAXF];
+};
+__global__ void __launch_bounds__(SB) k_feature_integrals(const Domain* dmp, const Sizing* zp,
+                                                          const __grid_constant__ IntegralPass ip, double* partial) {
+    __shared__ double ws[SB / 32];
+    int q = 0;
+    while (q + 1 < ip.n && (int)blockIdx.x >= ip.block0[q + 1]) ++q;
+    const Domain& dm = *dmp;
+    const Feat& f = dm.f[ip.k[q]];
+    const int block = blockIdx.x - ip.block0[q], nblocks = ip.block0[q + 1] - ip.block0[q], ln = ip.ln[q];
+    double acc = 0.0;
+    switch (f.kind) {
+        case SPH_FEAT_VOLUME: acc = integral_share<SPH_FEAT_VOLUME>(dm, *zp, f, ip.npts[q], ln, block, nblocks); break;
+        case SPH_FEAT_SEGMENT: acc = integral_share<SPH_FEAT_SEGMENT>(dm, *zp, f, ip.npts[q], ln, block, nblocks); break;
+        case SPH_FEAT_CIRCLE: acc = integral_share<SPH_FEAT_CIRCLE>(dm, *zp, f, ip.npts[q], ln, block, nblocks); break;
+        case SPH_FEAT_RECT: acc = integral_share<SPH_FEAT_RECT>(dm, *zp, f, ip.npts[q], ln, block, nblocks); break;
+        case SPH_FEAT_SPHERE: acc = integral_share<SPH_FEAT_SPHERE>(dm, *zp, f, ip.npts[q], ln, block, nblocks); break;
+        default: break;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -377,40 +421,40 @@ int quad_points(int kind, int D, long long* npts) {
 
 cudaError_t feature_integrals(const Domain& dm, const Domain* d_dom, const Sizing* d_siz, cudaStream_t st,
                               double* integral) {
-    // every feature's partial sums in one buffer, one copy back and one wait for all of them
+    // One launch, one copy back and one wait for all features: the curves and faces, each too small
+    // to fill the GPU, run beside the volume.  About 4,096 points per block of a small feature, and
+    // four blocks per SM for the largest.
     constexpr int NB = 4 * 152;
-    double* d_part = nullptr;
-    const size_t np = (size_t)NB * std::max(dm.nf, 1);
-    cudaError_t e = cudaMallocAsync(&d_part, sizeof(double) * np, st);
-    if (e != cudaSuccess) return e;
-    std::vector<double> part(np, 0.0);
-    e = cudaMemsetAsync(d_part, 0, sizeof(double) * np, st);
-    for (int k = 0; k < dm.nf && e == cudaSuccess; ++k) {
+    IntegralPass ip;
+    ip.n = 0;
+    ip.block0[0] = 0;
+    for (int k = 0; k < dm.nf; ++k) {
         if (dm.f[k].kind == SPH_FEAT_POINT) continue;
         long long npts = 0;
         const int nq = quad_points(dm.f[k].kind, dm.D, &npts);
+        if (npts == 0) continue;
         int ln = 0;
         while ((1 << ln) < nq) ++ln;
-        double* const out = d_part + (size_t)k * NB;
-        switch (dm.f[k].kind) {
-            case SPH_FEAT_VOLUME: k_feature_integral<SPH_FEAT_VOLUME><<<NB, SB, 0, st>>>(d_dom, d_siz, k, npts, ln, out); break;
-            case SPH_FEAT_SEGMENT: k_feature_integral<SPH_FEAT_SEGMENT><<<NB, SB, 0, st>>>(d_dom, d_siz, k, npts, ln, out); break;
-            case SPH_FEAT_CIRCLE: k_feature_integral<SPH_FEAT_CIRCLE><<<NB, SB, 0, st>>>(d_dom, d_siz, k, npts, ln, out); break;
-            case SPH_FEAT_RECT: k_feature_integral<SPH_FEAT_RECT><<<NB, SB, 0, st>>>(d_dom, d_siz, k, npts, ln, out); break;
-            case SPH_FEAT_SPHERE: k_feature_integral<SPH_FEAT_SPHERE><<<NB, SB, 0, st>>>(d_dom, d_siz, k, npts, ln, out); break;
-            default: break;
-        }
+        ip.k[ip.n] = k;
+        ip.ln[ip.n] = ln;
+        ip.npts[ip.n] = npts;
+        ip.block0[ip.n + 1] = ip.block0[ip.n] + (int)std::min<long long>(NB, (npts + 4095) / 4096);
+        ip.n += 1;
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(part.data(), d_part, sizeof(double) * np, cudaMemcpyDeviceToHost, st);
+    for (int k = 0; k < dm.nf; ++k) integral[k] = dm.f[k].kind == SPH_FEAT_POINT ? 1.0 : 0.0;
+    if (ip.n == 0) return cudaSuccess;
+    const int nb = ip.block0[ip.n];
+    double* d_part = nullptr;
+    cudaError_t e = cudaMallocAsync(&d_part, sizeof(double) * nb, st);
+    if (e != cudaSuccess) return e;
+    std::vector<double> part(nb, 0.0);
+    k_feature_integrals<<<nb, SB, 0, st>>>(d_dom, d_siz, ip, d_part);
+    e = cudaMemcpyAsync(part.data(), d_part, sizeof(double) * nb, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    for (int k = 0; k < dm.nf; ++k) {
-        if (dm.f[k].kind == SPH_FEAT_POINT) {
-            integral[k] = 1.0;
-            continue;
-        }
+    for (int q = 0; q < ip.n; ++q) {
         double sum = 0.0;
-        for (int b = 0; b < NB; ++b) sum += part[(size_t)k * NB + b];
-        integral[k] = sum;
+        for (int b = ip.block0[q]; b < ip.block0[q + 1]; ++b) sum += part[b];
+        integral[ip.k[q]] = sum;
     }
     cudaError_t f = cudaFreeAsync(d_part, st);
     if (e == cudaSuccess) e = f;

@@ -160,6 +160,10 @@ constexpr int LISTU = SPH_LISTU;
 // Measured, one kernel against three, us per step: the 2.6k square 48.6 against 52.2, a 20k disk
 // 77.2 against 79.8, a 120k disk 156.3 against 138.9; 3D, a 26k ball in three passes 372 against
 // 363.  In FP64 the neighbours' predictions cost more than the launches (2.9k square 116 against 110).
+// Six resident blocks per SM asked of the compiler: 20k disk 73.4 against 75.3 with four, 73.8 eight.
+#ifndef SPH_FUSED_MINB
+#define SPH_FUSED_MINB 6
+#endif
 #ifndef SPH_FUSED_MOST_2D
 #define SPH_FUSED_MOST_2D 32768
 #endif
@@ -169,7 +173,10 @@ constexpr int LISTU = SPH_LISTU;
 // resident one-warp blocks per SM asked of the compiler for the search (measured, 8 particles per
 // warp: 32 blocks at 64 registers with a few spills against 24 at 80, search and pressure pass of
 // the 1M disk 430 us against 461, of the 1.2M cube 1451 against 1552)
-constexpr int search_minb(int cl) { return cl == 16 ? 28 : 32; }
+#ifndef SPH_SEARCH_MINB_16
+#define SPH_SEARCH_MINB_16 28
+#endif
+constexpr int search_minb(int cl) { return cl == 16 ? SPH_SEARCH_MINB_16 : 32; }
 static_assert(CHUNK % (BLOCK / Lpp<2>::v) == 0 && CHUNK % (BLOCK / Lpp<3>::v) == 0,
               "a pair-pass block must lie in one chunk");
 // 3D occupancy cells finer than the cells-per-support top-level cells by 2^SPH_OCC_FINER per axis
