@@ -108,7 +108,7 @@ struct KTime {
 };
 // the step graph: rebuild = one-pass scan, scatter, gather (the keys and histogram come from
 // the previous step's update); interact = search, pressure pass; integrate = prediction, viscous
-// sum, update (which also computes the next keys)
+// sum, update (which also computes the next keys), one kernel for small batches
 constexpr int NSTAGE = 4;
 const KTime kStages[NSTAGE] = {{"rebuild", 3}, {"interact", 2}, {"control", 1}, {"integrate", 3}};
 // host copy of one instance
@@ -1588,7 +1588,7 @@ sph_status kernel_times_impl(sph_batch* b, sph_kernel_time* out, int32_t cap, in
     for (; k < NSTAGE && k < cap; ++k) {
         std::memset(out[k].name, 0, sizeof out[k].name);
         std::snprintf(out[k].name, sizeof out[k].name, "%s", kStages[k].name);
-        out[k].launches = b->stage_steps * kStages[k].kernels;
+        out[k].launches = b->stage_steps * (k == 3 && one_update_kernel(b->prec, b->D, b->nslots) ? 1 : kStages[k].kernels);
         out[k].total_ms = b->stage_ms[k];
     }
     if (n_out) *n_out = k;

@@ -830,7 +830,7 @@ template <typename T, int D>
 void launch_integrate(const State<T>& s, const One* one, const Ctrl* use, const Out<T>& o, cudaStream_t st,
                       bool pdl, int cls) {
     const int nb = div_up((long long)s.n * Lpp<D>::v, BLOCK), nu = div_up((long long)s.n, BLOCK);
-    if (sizeof(T) == 4 && s.n <= (D == 2 ? SPH_FUSED_MOST_2D : SPH_FUSED_MOST_3D)) {
+    if (one_update_kernel(sizeof(T) == 4 ? 32 : 64, D, s.n)) {
         if (one) launch_k(k_visc<T, D, true, true>, nb, BLOCK, st, pdl, s, *one, use, o, cls);
         else launch_k(k_visc<T, D, false, true>, nb, BLOCK, st, pdl, s, One(), use, o, cls);
     } else if (one) {

@@ -4,26 +4,29 @@
 
 namespace sph {
 
-// One warp per block: a block of several warps would hold its slots until the slowest of them is
-// done (neighbourhoods differ by the levels around).
+// One warp per block, two where a warp takes two particles (search_warps): a block holds its slots
+// until its slowest warp is done, and neighbourhoods differ by the levels around.
 // cls: the dimension class of the pass (in_pass), or -1 for every particle, whatever its dimension
 // or its instance's phase (inspection).  tested: if not null, the candidate pairs tested are
 // counted in it.
 template <typename T, int D, bool ONE, int CL>
-__global__ void __launch_bounds__(32, search_minb(CL)) k_search(State<T> s, One one, int cls, unsigned long long* tested) {
+__global__ void __launch_bounds__(32 * search_warps(CL), 32 / search_warps(CL))
+k_search(State<T> s, One one, int cls, unsigned long long* tested) {
     dep_launch();
     dep_wait();
-    constexpr int LPP = 32 / CL;
-    __shared__ SearchWarp<CL> ww;
+    constexpr int LPP = 32 / CL, WARPS = search_warps(CL);
+    static_assert(CHUNK % (CL * WARPS) == 0, "a block's slots lie in one chunk");
+    __shared__ SearchWarp<CL> sh[WARPS];
+    SearchWarp<CL>& ww = sh[WARPS == 1 ? 0 : threadIdx.x >> 5];
     __shared__ Grid gsh;
     __shared__ Params psh;
     const int lane = lane_id(), p = lane / LPP, sub = lane % LPP;
-    const int k0 = blockIdx.x * CL, k = k0 + p;
+    const int k0 = (blockIdx.x * WARPS + (WARPS == 1 ? 0 : threadIdx.x >> 5)) * CL, k = k0 + p;
     const int inst = ONE ? 0 : __ldg(s.chunk_inst + k0 / CHUNK);
     if (!ONE) {
         block_copy(&gsh, s.grids + inst);
         block_copy(&psh, s.params + inst);
-        __syncwarp();
+        __syncthreads();
     }
     const Grid& g = ONE ? one.g : gsh;
     const Params& prm = ONE ? one.p : psh;
@@ -54,14 +57,16 @@ __global__ void __launch_bounds__(32, search_minb(CL)) k_search(State<T> s, One 
 
 template <typename T, int D, int CL>
 void launch_search_cl(const State<T>& s, const One* one, cudaStream_t st, bool pdl, int cls, unsigned long long* tested) {
-    if (one) launch_k(k_search<T, D, true, CL>, div_up(s.n, CL), 32, st, pdl, s, *one, cls, tested);
-    else launch_k(k_search<T, D, false, CL>, div_up(s.n, CL), 32, st, pdl, s, One(), cls, tested);
+    const int nb = div_up(s.n, CL * search_warps(CL)), nt = 32 * search_warps(CL);
+    if (one) launch_k(k_search<T, D, true, CL>, nb, nt, st, pdl, s, *one, cls, tested);
+    else launch_k(k_search<T, D, false, CL>, nb, nt, st, pdl, s, One(), cls, tested);
 }
 template <typename T, int D>
 void launch_search(const State<T>& s, const One* one, cudaStream_t st, bool pdl, int cls, unsigned long long* tested) {
-    const int cl = SPH_SEARCH_CL ? SPH_SEARCH_CL : s.n <= SPH_SEARCH_N2 ? 2 : s.n <= SPH_SEARCH_N4 ? 4 : s.n <= SPH_SEARCH_N8 ? 8 : 16;
-    if (cl == 2) launch_search_cl<T, D, 2>(s, one, st, pdl, cls, tested);
-    else if (cl == 4) launch_search_cl<T, D, 4>(s, one, st, pdl, cls, tested);
+    const int cl = search_width(D, s.n);
+    if constexpr (D == 3)
+        if (cl == 2) return launch_search_cl<T, D, 2>(s, one, st, pdl, cls, tested);
+    if (cl == 4) launch_search_cl<T, D, 4>(s, one, st, pdl, cls, tested);
     else if (cl == 8) launch_search_cl<T, D, 8>(s, one, st, pdl, cls, tested);
     else launch_search_cl<T, D, 16>(s, one, st, pdl, cls, tested);
 }

@@ -133,29 +133,17 @@ template <int D> constexpr int list_entries() {
 }
 // consecutive list entries per lane and turn of the pair passes: their loads are in flight together
 // (measured on the 1.2M cube: 4 against 2 viscous sum and update 339 us against 468)
-#ifndef SPH_LISTU
-#define SPH_LISTU 4
-#endif
-constexpr int LISTU = SPH_LISTU;
-// particles searched by one warp: 2, 4, 8 or 16 by the slots of the batch (up to N2, N4, N8 slots).
+constexpr int LISTU = 4;
+// particles searched by one warp: 2 (in 3D), 4, 8 or 16 by the slots of the batch.
 // A warp searching for more particles reads the cells around them once for all, one searching for
 // fewer is done sooner, which counts while the GPU is not full.  The lists do not depend on it.
 // Measured, search and pressure pass in us with 2 / 4 / 8 / 16: a 26k ball in three passes (whole
 // step) 376 / 437 / 640 / 826; a 20k disk 33 / 29 / 38 / 55; 120k disk 106 / 76 / 66 / 79; 1M disk
 // - / - / 430 / 404; 83k cube 189 / 149 / 137 / 146; 300k cube 671 / 498 / 472 / -; 1.2M cube
 // 2447 / - / 1451 / 1408.
-#ifndef SPH_SEARCH_CL
-#define SPH_SEARCH_CL 0
-#endif
-#ifndef SPH_SEARCH_N2
-#define SPH_SEARCH_N2 (D == 3 ? 32768 : 0)
-#endif
-#ifndef SPH_SEARCH_N4
-#define SPH_SEARCH_N4 65536
-#endif
-#ifndef SPH_SEARCH_N8
-#define SPH_SEARCH_N8 524288
-#endif
+constexpr int search_width(int D, int slots) {
+    return D == 3 && slots <= 32768 ? 2 : slots <= 65536 ? 4 : slots <= 524288 ? 8 : 16;
+}
 // most slots of a batch whose prediction, viscous sum and update run as one kernel (FP32 build).
 // Measured, one kernel against three, us per step: the 2.6k square 48.6 against 52.2, a 20k disk
 // 77.2 against 79.8, a 120k disk 156.3 against 138.9; 3D, a 26k ball in three passes 372 against
@@ -170,13 +158,16 @@ constexpr int LISTU = SPH_LISTU;
 #ifndef SPH_FUSED_MOST_3D
 #define SPH_FUSED_MOST_3D 8192
 #endif
-// resident one-warp blocks per SM asked of the compiler for the search (measured, 8 particles per
-// warp: 32 blocks at 64 registers with a few spills against 24 at 80, search and pressure pass of
-// the 1M disk 430 us against 461, of the 1.2M cube 1451 against 1552)
-#ifndef SPH_SEARCH_MINB_16
-#define SPH_SEARCH_MINB_16 28
-#endif
-constexpr int search_minb(int cl) { return cl == 16 ? SPH_SEARCH_MINB_16 : 32; }
+inline bool one_update_kernel(int precision, int D, int slots) {
+    return precision == 32 && slots <= (D == 2 ? SPH_FUSED_MOST_2D : SPH_FUSED_MOST_3D);
+}
+// Warps per block of the search, and 32 resident warps per SM asked of the compiler (64 registers
+// with a few spills).  Measured, us per step: 16 particles per warp at 20, 24, 28, 32 resident warps
+// 701, 664, 655, 646 on the 1M disk, 2104, 1991, 1925, 1869 on the 1.2M cube; two-warp blocks there
+// 688 and 2011 (a block's slots wait for its slower warp), at 36 and 40 resident warps 674..682 and
+// 1966..2009 (spills).  Where a warp takes two particles its work is short and the launch of the
+// blocks weighs more than the wait: two warps 270 against 280 on a 26k ball in lattice order.
+constexpr int search_warps(int cl) { return cl == 2 ? 2 : 1; }
 static_assert(CHUNK % (BLOCK / Lpp<2>::v) == 0 && CHUNK % (BLOCK / Lpp<3>::v) == 0,
               "a pair-pass block must lie in one chunk");
 // 3D occupancy cells finer than the cells-per-support top-level cells by 2^SPH_OCC_FINER per axis
