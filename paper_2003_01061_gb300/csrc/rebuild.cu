@@ -26,7 +26,8 @@ template <typename T, int D, bool ONE> __global__ void __launch_bounds__(BLOCK) 
     atomicAdd(s.count + key, 1);
 }
 
-// ---- exclusive scan of the per-cell counts: three passes over tiles of SCAN_TILE cells ----
+// ---- exclusive scan of the per-cell counts, in one pass (steps) or in three passes over tiles of
+// SCAN_TILE cells (callers without scratch for the look-back) ----
 __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int& total) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int x = v;

@@ -138,10 +138,6 @@ __device__ __forceinline__ double rn_mul(double a, double b) { return __dmul_rn(
 
 __device__ __forceinline__ unsigned long long min_bits(float v) { return (unsigned long long)__float_as_uint(v); }
 __device__ __forceinline__ unsigned long long min_bits(double v) { return (unsigned long long)__double_as_longlong(v); }
-// a working-precision value as a float not below it
-template <typename T> __device__ __forceinline__ float float_up(T v);
-template <> __device__ __forceinline__ float float_up<float>(float v) { return v; }
-template <> __device__ __forceinline__ float float_up<double>(double v) { return __double2float_ru(v); }
 template <typename T> __device__ __forceinline__ T from_bits(unsigned long long b);
 template <> __device__ __forceinline__ float from_bits<float>(unsigned long long b) { return __uint_as_float((unsigned)b); }
 template <> __device__ __forceinline__ double from_bits<double>(unsigned long long b) { return __longlong_as_double((long long)b); }

@@ -91,19 +91,12 @@ __device__ __forceinline__ void list_load(const float* p, float (&f)[4]) {
     const float4 v = *reinterpret_cast<const float4*>(p);
     f[0] = v.x, f[1] = v.y, f[2] = v.z, f[3] = v.w;
 }
-__device__ __forceinline__ void list_load(const float* p, float (&f)[2]) {
-    const float2 v = *reinterpret_cast<const float2*>(p);
-    f[0] = v.x, f[1] = v.y;
-}
 template <int U> __device__ __forceinline__ void list_store(double* p, const double (&f)[U]) {
 #pragma unroll
     for (int u = 0; u < U; ++u) p[u] = f[u];
 }
 __device__ __forceinline__ void list_store(float* p, const float (&f)[4]) {
     *reinterpret_cast<float4*>(p) = make_float4(f[0], f[1], f[2], f[3]);
-}
-__device__ __forceinline__ void list_store(float* p, const float (&f)[2]) {
-    *reinterpret_cast<float2*>(p) = make_float2(f[0], f[1]);
 }
 
 // ---- the search of one warp ----
