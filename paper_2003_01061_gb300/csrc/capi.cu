@@ -506,7 +506,7 @@ template <typename T> void set_slots(sph_batch* b) {
 // count changes).  Slot ranges: the loaded instances in index order, each its count rounded up
 // to CHUNK; the stored state of every other loaded instance is moved to its new range on the
 // device.  Key ranges: each loaded instance's cells and its dummy key.  The per-cell arrays are
-// reallocated if too small and cleared (the relative scan then starts from zero counts).
+// reallocated if too small and cleared (the histogram starts from zero counts).
 // Uploads the grids and the descriptors of instance `desc` (all instances for desc < 0).
 // Fails with SPH_E_NOMEM, changing nothing, when the slots do not fit the allocation.
 sph_status relayout(sph_batch* b, int changed, int new_n, int desc) {

@@ -53,35 +53,21 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int& 
     return before + x - v;
 }
 
-// relative: the counters were not reset since the previous rebuild, where the scatter left
-// count[c] = cell_start[c+1]; the new per-cell count is count[c] - cell_start[c+1] (and is
-// stored back into count for the down-sweep), so no pass over all cells resets them.
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(int ncell, int* __restrict__ count,
-                                                              const int* __restrict__ cell_start, bool relative,
-                                                              int* __restrict__ bsum) {
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(int ncell, const int* __restrict__ count, int* __restrict__ bsum) {
     __shared__ int ws[32];
     int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
     int v = 0;
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; ++k)
-        if (base + k < ncell) {
-            int nk = count[base + k];
-            if (relative) {
-                nk -= cell_start[base + k + 1];
-                count[base + k] = nk;
-            }
-            v += nk;
-        }
+        if (base + k < ncell) v += count[base + k];
     int total;
     block_exclusive_scan(v, ws, total);
     if (threadIdx.x == 0) bsum[blockIdx.x] = total;
 }
 
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_top(int nb, int ncell, int* __restrict__ bsum,
-                                                           int* __restrict__ cell_start, unsigned* __restrict__ occ,
-                                                           int nocc) {
+                                                           int* __restrict__ cell_start) {
     __shared__ int ws[32];
-    for (int t = threadIdx.x; t < nocc * OCCW; t += blockDim.x) occ[t] = 0u;   // rebuilt by the gather
     int base = threadIdx.x * SCAN_ITEMS;
     int loc[SCAN_ITEMS];
     int v = 0;
@@ -126,13 +112,13 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(int ncell, int* __re
 
 // ---- the step's scan in one pass: decoupled look-back ----
 // Every block takes the next tile by ticket (so all tiles before it are running or done),
-// computes its counts (relative: count[c] - cell_start[c+1], the previous scatter having left
-// count[c] = cell_start[c+1]) and their sum, publishes the sum, then walks back over the
-// preceding tiles' words (32 at a time, one per lane of its first warp) until it meets a
-// published inclusive prefix, publishes its own
-// inclusive prefix and writes cell_start and the scatter cursors of its cells.  A tile reads
-// the old cell_start[c+1] of its last cell (the next tile's first) before it publishes its
-// sum, and the next tile writes it only after it has seen that sum, so the read comes first.
+// sums its counts, publishes the sum, then walks back over the preceding tiles' words (32 at a
+// time, one per lane of its first warp) until it meets a published inclusive prefix, publishes its
+// own inclusive prefix and writes cell_start.  It reads 4 bytes per cell and writes 4: the counts
+// need no reset, since the scatter takes them down to zero (with cursors left in their place, reset
+// by subtracting the old cell_start, 8 and 8 bytes: rebuild of the 12M cells of the 83k graded cube 73
+// us against 62, of the 1M disk 83 against 74).  Looking back over 128 or 256 tiles at once instead
+// of 32 was slower (58 and 62 us against 55 at 8 cells per thread).
 // Spins are bounded: a tile that waits too long records ST_SCAN and goes on (the walks and the
 // gather clamp every cell range, so the step stays in bounds; the host reports the error).
 constexpr unsigned long long TS_AGG = 1ull << 62, TS_PRE = 2ull << 62, TS_VAL = 0xffffffffull;
@@ -154,21 +140,14 @@ template <typename T> __global__ void __launch_bounds__(SCAN1_THREADS) k_scan_on
     int v = 0;
     if (whole) {
         const int4* const cn = reinterpret_cast<const int4*>(s.count + base);
-        const int4* const cs = reinterpret_cast<const int4*>(s.cell_start + base);
-        int old[SCAN1_ITEMS + 1];
-        old[SCAN1_ITEMS] = s.cell_start[base + SCAN1_ITEMS];
 #pragma unroll
         for (int k = 0; k < SCAN1_ITEMS / 4; ++k) {
-            const int4 c = cn[k], o = cs[k];
+            const int4 c = cn[k];
             loc[4 * k] = c.x, loc[4 * k + 1] = c.y, loc[4 * k + 2] = c.z, loc[4 * k + 3] = c.w;
-            old[4 * k] = o.x, old[4 * k + 1] = o.y, old[4 * k + 2] = o.z, old[4 * k + 3] = o.w;
         }
-#pragma unroll
-        for (int k = 0; k < SCAN1_ITEMS; ++k) loc[k] -= old[k + 1];
     } else {
 #pragma unroll
-        for (int k = 0; k < SCAN1_ITEMS; ++k)
-            loc[k] = base + k < ncell ? s.count[base + k] - s.cell_start[base + k + 1] : 0;
+        for (int k = 0; k < SCAN1_ITEMS; ++k) loc[k] = base + k < ncell ? s.count[base + k] : 0;
     }
 #pragma unroll
     for (int k = 0; k < SCAN1_ITEMS; ++k) v += loc[k];
@@ -217,25 +196,19 @@ template <typename T> __global__ void __launch_bounds__(SCAN1_THREADS) k_scan_on
     __syncthreads();
     ex += sh_prefix;
 #pragma unroll
-    for (int k = 0; k < SCAN1_ITEMS; ++k) {   // loc: the start of the cell, also its scatter cursor
+    for (int k = 0; k < SCAN1_ITEMS; ++k) {   // loc: the start of the cell
         const int n = loc[k];
         loc[k] = ex;
         ex += n;
     }
     if (whole) {
 #pragma unroll
-        for (int k = 0; k < SCAN1_ITEMS / 4; ++k) {
-            const int4 e = make_int4(loc[4 * k], loc[4 * k + 1], loc[4 * k + 2], loc[4 * k + 3]);
-            reinterpret_cast<int4*>(s.cell_start + base)[k] = e;
-            reinterpret_cast<int4*>(s.count + base)[k] = e;
-        }
+        for (int k = 0; k < SCAN1_ITEMS / 4; ++k)
+            reinterpret_cast<int4*>(s.cell_start + base)[k] = make_int4(loc[4 * k], loc[4 * k + 1], loc[4 * k + 2], loc[4 * k + 3]);
     } else {
 #pragma unroll
         for (int k = 0; k < SCAN1_ITEMS; ++k)
-            if (base + k < ncell) {
-                s.cell_start[base + k] = loc[k];
-                s.count[base + k] = loc[k];
-            }
+            if (base + k < ncell) s.cell_start[base + k] = loc[k];
     }
     if (base + SCAN1_ITEMS >= ncell && base < ncell) s.cell_start[ncell] = ex;   // the thread holding the last cell
 }
@@ -247,12 +220,13 @@ template <typename T> __global__ void __launch_bounds__(BLOCK) k_scatter(State<T
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= s.n) return;
     const int key = s.K[i];
-    // one atomic per cell present in the warp (sorted neighbours mostly share cells); each
-    // lane takes the cursor plus its rank among the lanes of its cell
+    // one atomic per cell present in the warp (sorted neighbours mostly share cells): it takes the
+    // lanes of a cell off the cell's count, and they fill the places from there up.  Every count
+    // ends at zero, ready for the next step's histogram
     const unsigned peers = __match_any_sync(__activemask(), key);
     const int lane = threadIdx.x & 31, lead = __ffs(peers) - 1;
     int pos = 0;
-    if (lane == lead) pos = atomicAdd(s.count + key, __popc(peers));
+    if (lane == lead) pos = s.cell_start[key] + atomicSub(s.count + key, __popc(peers)) - __popc(peers);
     pos = __shfl_sync(peers, pos, lead) + __popc(peers & ((1u << lane) - 1u));
     if ((unsigned)pos < (unsigned)s.n) {
         s.perm[pos] = i;
@@ -431,11 +405,10 @@ template <typename T, int D> void launch_hash(const State<T>& s, const One* one,
     if (one) k_hash<T, D, true><<<div_up(s.n, BLOCK), BLOCK, 0, st>>>(s, *one);
     else k_hash<T, D, false><<<div_up(s.n, BLOCK), BLOCK, 0, st>>>(s, One());
 }
-void launch_scan(int ncell, int* count, int* cell_start, int* bsum, cudaStream_t st, unsigned* occ, int nocc,
-                 bool relative) {
+void launch_scan(int ncell, int* count, int* cell_start, int* bsum, cudaStream_t st) {
     int nb = div_up(ncell, SCAN_TILE);
-    k_scan_reduce<<<nb, SCAN_THREADS, 0, st>>>(ncell, count, cell_start, relative, bsum);
-    k_scan_top<<<1, SCAN_THREADS, 0, st>>>(nb, ncell, bsum, cell_start, occ, nocc);
+    k_scan_reduce<<<nb, SCAN_THREADS, 0, st>>>(ncell, count, bsum);
+    k_scan_top<<<1, SCAN_THREADS, 0, st>>>(nb, ncell, bsum, cell_start);
     k_scan_down<<<nb, SCAN_THREADS, 0, st>>>(ncell, count, bsum, cell_start);
 }
 template <typename T> void launch_scan_onepass(const State<T>& s, cudaStream_t st) {

@@ -45,7 +45,7 @@ template <typename T> struct State {
     Vec4<T>* P;
     float4* F;         // search records: position and kappa h / 2 in finest cells (padding: stale)
     Vec4<T>* A;
-    // rebuild scratch: per-cell counts (also the scatter cursors), cell starts, scan block
+    // rebuild scratch: per-cell counts (down to zero after the scatter), cell starts, scan block
     // sums, and the sorted-slot -> stored-index permutation
     int* count;
     int* cell_start;
@@ -279,12 +279,12 @@ constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_ITEMS = 4;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
 // cells per thread (read and written as 16-byte words) and threads per tile of the step's one-pass
-// scan (bound by DRAM and the tiles' chain: 200 MB in 45 us on the 12M cells of the 83k graded cube;
-// measured, rebuild in us, 2 cells per thread word by word / 4 / 8 / 8 with 512 threads: 20k disk
-// 16.5 / 16.2 / 17.6 / 16.3, 1M disk 111 / 84.6 / 83.7 / 82.9, 83k cube 105 / 73.2 / 72.3 / 72.4, 1.2M
-// cube 106 / 90.0 / 91.2 / 90.3)
+// scan (bound by DRAM and the tiles' chain: 100 MB on the 12M cells of the 83k graded cube; measured,
+// rebuild in us, 4 cells per thread / 8 / 16 / 8 with 512 threads: 20k disk 15.6 / 16.0 / 18.2 / 15.9,
+// 1M disk 73.8 / 66.9 / 66.0 / 67.5, 83k cube 62.2 / 55.1 / 53.6 / 54.7, 1.2M cube 82.6 / 79.2 / 79.0 /
+// 79.0)
 #ifndef SPH_SCAN1_ITEMS
-#define SPH_SCAN1_ITEMS 4
+#define SPH_SCAN1_ITEMS 8
 #endif
 #ifndef SPH_SCAN1_THREADS
 #define SPH_SCAN1_THREADS 1024
@@ -326,9 +326,8 @@ inline void launch_k(void (*kern)(K...), int grid, int block, cudaStream_t st, b
 // rebuild.cu
 // `one`: the descriptors of a batch of one (nullptr: read the per-instance tables)
 template <typename T, int D> void launch_hash(const State<T>& s, const One* one, cudaStream_t st);
-void launch_scan(int ncell, int* count, int* cell_start, int* bsum, cudaStream_t st, unsigned* occ = nullptr,
-                 int nocc = 0, bool relative = false);
-// relative one-pass scan of the step (decoupled look-back over tiles taken in ticket order)
+void launch_scan(int ncell, int* count, int* cell_start, int* bsum, cudaStream_t st);
+// one-pass scan of the step (decoupled look-back over tiles taken in ticket order)
 template <typename T> void launch_scan_onepass(const State<T>& s, cudaStream_t st);
 template <typename T> void launch_scatter(const State<T>& s, cudaStream_t st, bool pdl = false);
 void launch_cellsort(int ncell, int n, const int* cell_start, int* perm, int* count, cudaStream_t st);
