@@ -226,31 +226,11 @@ __device__ __forceinline__ bool inside(const Domain& dm, const double x[3], cons
     return samp_phi(dm, x) > 0.0;
 }
 
-// sqrt(s) of a normal s: the hardware's estimate of 1/sqrt and one third-order step of Newton's
-// iteration (e = 1 - s y^2, sqrt = s y (1 + e/2 + 3/8 e^2)), within an ulp; the acceptance test of
-// the sampling keeps the correctly rounded root
-__device__ __forceinline__ double quad_root(double s) {
-    if (!(s > 1e-280 && s < 1e280)) return sqrt(s);
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
-    const double t = s * y, e = fma(-t, y, 1.0);
-    return fma(t * e, fma(0.375, e, 0.5), t);
-}
-
-// h_t(x) as samp_h has it but for the rounding of the root, and without the FP64 roots of reference circles and spheres that single
-// precision shows to be clearly farther than the nearest one.
+// h_t(x) of a point of the volume, bit for bit as samp_h has it: with several reference circles or
+// spheres, only the nearest one's distance is formed in FP64 where single precision shows which it
+// is (by far more than its rounding, 2^-20 of the domain's size).
 __device__ __forceinline__ double quad_h(const Sizing& z, const double x[3], const float xf[3], float size) {
-    auto root_dist = [&](const double* c) {
-        const double d0 = x[0] - c[0], d1 = x[1] - c[1], d2 = x[2] - c[2];
-        return quad_root(fma(d2, d2, fma(d1, d1, d0 * d0)));
-    };
-    auto clamp = [&](double h) {
-        if (h < z.lo) h = z.lo;
-        return h > z.hi ? z.hi : h;
-    };
-    if (z.kind == 2) return clamp(z.a + z.b * root_dist(z.q));
-    if (z.kind != 1 || z.nref < 1) return samp_h(z, x);
-    if (z.nref == 1) return clamp(z.a + z.b * fabs(root_dist(z.rc[0]) - z.rr[0]));
+    if (z.kind != 1 || z.nref < 2) return samp_h(z, x);
     float best = 3e38f, next = 3e38f;
     int kb = 0;
     for (int k = 0; k < z.nref; ++k) {
@@ -266,18 +246,27 @@ __device__ __forceinline__ double quad_h(const Sizing& z, const double x[3], con
         }
     }
     if (!(next - best > size * 0x1p-16f)) return samp_h(z, x);
-    return clamp(z.a + z.b * fabs(root_dist(z.rc[kb]) - z.rr[kb]));
+    double h = dadd(z.a, dmul(z.b, fabs(dsub(dist_n(x, z.rc[kb], 3), z.rr[kb]))));
+    if (h < z.lo) h = z.lo;
+    if (h > z.hi) h = z.hi;
+    return h;
 }
 
 // Midpoint-rule integral of rho_t over feature k (Eqs. 10, 11), per-block partial sums.  The
 // quadrature sizes are powers of two (nq = 2^ln), so the divisions by nq are exact and a point's
 // indices are bits of its number; what does not depend on the point is computed before the loop.
+// Where a feature's measure over h^d is an odd multiple of 1/2 (constant spacing) the rounding of
+// the terms and the order of their sum decide the rounded count: the terms use correctly rounded
+// roots and quotients, and every feature is summed over the same QUAD_BLOCKS blocks of SB threads
+// whatever its size.  (Roots and reciprocals by one Newton step, within an ulp, and fewer blocks for
+// the small features gave other counts in 14 of 821 such features.)
 // Bound by the FP64 pipe, two multiply-adds per SM and clock: a volume point costs one root and one
-// reciprocal (about 30 FP64 instructions), where three quotients for the cell size and a second
-// root for the level set made it about 130.
+// quotient.  All features of a cube take 2.19 ms, of a disk 0.43 (one launch per feature, with
+// quotients per point for the cell size and a second root for the level set: 4.41 and 1.49).
+constexpr int QUAD_BLOCKS = 4 * 152;
 template <int KIND>
 __device__ __forceinline__ double integral_share(const Domain& dm, const Sizing& z, const Feat& f, long long npts, int ln,
-                                                 int block, int nblocks) {
+                                                 int block) {
     const int D = dm.D, nq = 1 << ln, last = nq - 1;
     const double inq = 1.0 / nq;
     float size = 0.0f;   // of the domain, with its distance from the origin
@@ -305,7 +294,7 @@ __device__ __forceinline__ double integral_share(const Domain& dm, const Sizing&
     if (KIND == SPH_FEAT_CIRCLE) cell = 2.0 * CUDART_PI * f.g[2] * inq;
     if (KIND == SPH_FEAT_RECT) cell = (f.g[9] * inq) * (f.g[10] * inq);
     double acc = 0.0;
-    for (long long i = (long long)block * SB + threadIdx.x; i < npts; i += (long long)nblocks * SB) {
+    for (long long i = (long long)block * SB + threadIdx.x; i < npts; i += (long long)QUAD_BLOCKS * SB) {
         double x[3] = {0.0, 0.0, 0.0};
         if (KIND == SPH_FEAT_VOLUME) {
             float xf[3];
@@ -315,25 +304,22 @@ __device__ __forceinline__ double integral_share(const Domain& dm, const Sizing&
             }
             if (inside(dm, x, xf, size)) {
                 const double h = quad_h(z, x, xf, size);
-                acc += cell * fast_rcp(D == 3 ? h * h * h : h * h);
+                acc += cell / (D == 3 ? h * h * h : h * h);
             }
         } else if (KIND == SPH_FEAT_SEGMENT) {
             const double t = (i + 0.5) * inq;
             for (int a = 0; a < 3; ++a) x[a] = f.g[a] + t * dx[a];
-            const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
-            acc += cell / quad_h(z, x, xf, size);
+            acc += cell / samp_h(z, x);
         } else if (KIND == SPH_FEAT_CIRCLE) {
             const double th = 2.0 * CUDART_PI * (i + 0.5) * inq;
             x[0] = f.g[0] + f.g[2] * cos(th);
             x[1] = f.g[1] + f.g[2] * sin(th);
-            const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
-            acc += cell / quad_h(z, x, xf, size);
+            acc += cell / samp_h(z, x);
         } else if (KIND == SPH_FEAT_RECT) {
             const double si = (((int)i & last) + 0.5) * inq * f.g[9], tj = ((int)(i >> ln) + 0.5) * inq * f.g[10];
             for (int a = 0; a < 3; ++a) x[a] = f.g[a] + si * f.g[3 + a] + tj * f.g[6 + a];
-            const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
-            const double h = quad_h(z, x, xf, size);
-            acc += cell * fast_rcp(h * h);
+            const double h = samp_h(z, x);
+            acc += cell / (h * h);
         } else if (KIND == SPH_FEAT_SPHERE) {
             const int ii = (int)(i >> (ln + 1)), jj = (int)i & (2 * nq - 1);
             const double th = CUDART_PI * (ii + 0.5) * inq, ph = CUDART_PI * (jj + 0.5) * inq;
@@ -344,8 +330,7 @@ __device__ __forceinline__ double integral_share(const Domain& dm, const Sizing&
             x[0] = f.g[0] + R * st * cp;
             x[1] = f.g[1] + R * st * sp;
             x[2] = f.g[2] + R * ct;
-            const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
-            const double h = quad_h(z, x, xf, size);
+            const double h = samp_h(z, x);
             acc += R * R * st * (CUDART_PI * inq) * (CUDART_PI * inq) / (h * h);
         }
     }
@@ -365,14 +350,14 @@ __global__ void __launch_bounds__(SB) k_feature_integrals(const Domain* dmp, con
     while (q + 1 < ip.n && (int)blockIdx.x >= ip.block0[q + 1]) ++q;
     const Domain& dm = *dmp;
     const Feat& f = dm.f[ip.k[q]];
-    const int block = blockIdx.x - ip.block0[q], nblocks = ip.block0[q + 1] - ip.block0[q], ln = ip.ln[q];
+    const int block = blockIdx.x - ip.block0[q], ln = ip.ln[q];
     double acc = 0.0;
     switch (f.kind) {
-        case SPH_FEAT_VOLUME: acc = integral_share<SPH_FEAT_VOLUME>(dm, *zp, f, ip.npts[q], ln, block, nblocks); break;
-        case SPH_FEAT_SEGMENT: acc = integral_share<SPH_FEAT_SEGMENT>(dm, *zp, f, ip.npts[q], ln, block, nblocks); break;
-        case SPH_FEAT_CIRCLE: acc = integral_share<SPH_FEAT_CIRCLE>(dm, *zp, f, ip.npts[q], ln, block, nblocks); break;
-        case SPH_FEAT_RECT: acc = integral_share<SPH_FEAT_RECT>(dm, *zp, f, ip.npts[q], ln, block, nblocks); break;
-        case SPH_FEAT_SPHERE: acc = integral_share<SPH_FEAT_SPHERE>(dm, *zp, f, ip.npts[q], ln, block, nblocks); break;
+        case SPH_FEAT_VOLUME: acc = integral_share<SPH_FEAT_VOLUME>(dm, *zp, f, ip.npts[q], ln, block); break;
+        case SPH_FEAT_SEGMENT: acc = integral_share<SPH_FEAT_SEGMENT>(dm, *zp, f, ip.npts[q], ln, block); break;
+        case SPH_FEAT_CIRCLE: acc = integral_share<SPH_FEAT_CIRCLE>(dm, *zp, f, ip.npts[q], ln, block); break;
+        case SPH_FEAT_RECT: acc = integral_share<SPH_FEAT_RECT>(dm, *zp, f, ip.npts[q], ln, block); break;
+        case SPH_FEAT_SPHERE: acc = integral_share<SPH_FEAT_SPHERE>(dm, *zp, f, ip.npts[q], ln, block); break;
         default: break;
     }
 #pragma unroll
@@ -389,7 +374,7 @@ __global__ void __launch_bounds__(SB) k_feature_integrals(const Domain* dmp, con
 constexpr bool power_of_two(int n) { return n > 0 && (n & (n - 1)) == 0; }
 static_assert(power_of_two(SPH_QUAD_AREA) && power_of_two(SPH_QUAD_VOLUME) && power_of_two(SPH_QUAD_CURVE) &&
                   power_of_two(SPH_QUAD_FACE) && power_of_two(SPH_QUAD_SPHERE),
-              "k_feature_integral takes a point's indices from the bits of its number");
+              "integral_share takes a point's indices from the bits of its number");
 
 }  // namespace
 
@@ -422,9 +407,7 @@ int quad_points(int kind, int D, long long* npts) {
 cudaError_t feature_integrals(const Domain& dm, const Domain* d_dom, const Sizing* d_siz, cudaStream_t st,
                               double* integral) {
     // One launch, one copy back and one wait for all features: the curves and faces, each too small
-    // to fill the GPU, run beside the volume.  About 4,096 points per block of a small feature, and
-    // four blocks per SM for the largest.
-    constexpr int NB = 4 * 152;
+    // to fill the GPU, run beside the volume.  Blocks without a point are left out (their sums are 0).
     IntegralPass ip;
     ip.n = 0;
     ip.block0[0] = 0;
@@ -438,7 +421,7 @@ cudaError_t feature_integrals(const Domain& dm, const Domain* d_dom, const Sizin
         ip.k[ip.n] = k;
         ip.ln[ip.n] = ln;
         ip.npts[ip.n] = npts;
-        ip.block0[ip.n + 1] = ip.block0[ip.n] + (int)std::min<long long>(NB, (npts + 4095) / 4096);
+        ip.block0[ip.n + 1] = ip.block0[ip.n] + (int)std::min<long long>(QUAD_BLOCKS, (npts + SB - 1) / SB);
         ip.n += 1;
     }
     for (int k = 0; k < dm.nf; ++k) integral[k] = dm.f[k].kind == SPH_FEAT_POINT ? 1.0 : 0.0;
