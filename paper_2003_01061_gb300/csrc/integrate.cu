@@ -591,8 +591,7 @@ __device__ __noinline__ void visc_again(const State<T>& s, const Grid& g, const 
                 if (meta_group(MetaWord<D>::meta(w)) != gi || !(r2 < pair_rc2(hi, hj, hk)) || !(r2 > T(0))) continue;
                 hpow(hj, di, hjd, hj2d);
                 const Vec4<T> q = FUSED ? predicted<T>(p, StepOf<T>(p, cu, gi), s.A[j], s.VH[j], di) : s.A[j];
-                visc_pair<T, D>(me, q,
-                                (hi2d + hj2d) * wendland_slope<T>(di, root_of(r2), fast_rcp(hk * (hi + hj))), sum);
+                visc_pair<T, D>(me, q, kernel_factor<T>(di, hi2d + hj2d, root_of(r2), fast_rcp(hk * (hi + hj))), sum);
             }
         });
     for (int a = 0; a < 3; ++a) av[a] += sum[a];

@@ -134,7 +134,7 @@ template <typename T, int D> struct Pressure {
             const T w4 = (q * q) * (q * q) * (T(5) - T(4) * q);   // (1 - r/R)^4 (1 + 4 r/R)
             sig += w4;
             gam += w4 * hjd;
-            const T kv = S2 * wendland_slope<T>(di, r, fast_rcp(R));
+            const T kv = kernel_factor<T>(di, S2, r, fast_rcp(R));
             for (int a = 0; a < D; ++a) F[a] += kv * dx[a];
             return near && r2 > T(0) ? kv : T(0);
         }
@@ -318,8 +318,8 @@ __global__ void __launch_bounds__(BLOCK, (interact_minb<T, D>()))
                     q = fma2(r, neg2(invR), one2);
                     unpack2(q, xa, xb);
                     q = pack2(sa ? fmaxf(xa, 0.0f) : 0.0f, sb ? fmaxf(xb, 0.0f) : 0.0f);
-                    const f32x2 i2 = mul2(invR, invR), i4 = mul2(i2, i2);
-                    const f32x2 kv = mul2(mul2(S2, mul2(pick(mul2(i2, invR), i4, mul2(i4, invR)), A2)), mul2(mul2(q, q), q));
+                    const f32x2 i2 = mul2(invR, invR);   // products in the order of kernel_factor
+                    const f32x2 kv = mul2(mul2(mul2(S2, i2), mul2(pick(invR, i2, mul2(i2, invR)), A2)), mul2(mul2(q, q), q));
                     F0 = fma2(kv, dx, F0);
                     F1 = fma2(kv, dy, F1);
                     if (D == 3) F2 = fma2(kv, dz, F2);

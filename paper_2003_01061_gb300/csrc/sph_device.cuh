@@ -489,16 +489,14 @@ __device__ __forceinline__ double root_of(double v) { return sqrt(v); }
 __device__ __forceinline__ float pos_part(float v) { return fmaxf(v, 0.0f); }
 __device__ __forceinline__ double pos_part(double v) { return fmax(v, 0.0); }
 
-// W'(r)/r of the Wendland C2 kernel with support 1/invR in d dimensions: -20 alpha_d (1-q)^3 / R^2,
-// zero outside the support
-template <typename T> __device__ __forceinline__ T wendland_slope(int d, T r, T invR) {
-    const T t = pos_part(T(1) - r * invR);
-    if constexpr (sizeof(T) == 8) {   // fewer products: A_d / R^(d+2)
-        const T i2 = invR * invR, i3 = i2 * invR;
-        const T a = d == 1 ? T(-30) * i3 : d == 2 ? T(-140.0 / CUDART_PI) * (i2 * i2) : T(-210.0 / CUDART_PI) * (i2 * i3);
-        return a * (t * t * t);
-    }
-    return (wendland_alpha<T>(d, invR) * (T(-20) * invR * invR)) * (t * t * t);
+// The kernel factor of a pair, S2 W'(r)/r for the Wendland C2 kernel with support 1/invR in d
+// dimensions and S2 = rho_i^-2 + rho_j^-2: -20 alpha_d S2 (1-q)^3 / R^2, zero outside the support.
+// S2 ~ h^(2d) meets part of R^-(d+2) first: alone, that power leaves the single-precision range for
+// 2D spacings below 2e-10, where S2 is still a number.
+template <typename T> __device__ __forceinline__ T kernel_factor(int d, T S2, T r, T invR) {
+    const T t = pos_part(T(1) - r * invR), i2 = invR * invR;
+    const T a = d == 1 ? T(-30) * invR : d == 2 ? T(-140.0 / CUDART_PI) * i2 : T(-210.0 / CUDART_PI) * (i2 * invR);
+    return (S2 * i2) * a * (t * t * t);
 }
 
 // sum over the LPP lanes of one particle (xor butterfly: every lane gets the same bits).  The
