@@ -542,13 +542,6 @@ __global__ void __launch_bounds__(BLOCK) k_predict(State<T> s, One one, const Ct
     if (moves(p, use + inst, gi, di, cls, D)) s.A[k] = predicted<T>(p, StepOf<T>(p, use + inst, gi), a, vh, di);
 }
 
-// 2 a b / (a + b) for a, b >= 0 (0 where the sum is 0)
-template <typename T> __device__ __forceinline__ T harmonic(T a, T b) {
-    const T s = a + b;
-    if (sizeof(T) == 8 && s > T(1e-280)) return T(2) * a * b * fast_rcp(s);   // s far from the range's end
-    return s > T(0) ? T(2) * a * b / s : T(0);
-}
-
 // the viscous term of Eq. 7 of a pair: me, q the two particles' (v~, eta), kv the kernel factor
 template <typename T, int D> __device__ __forceinline__ void visc_pair(const Vec4<T>& me, const Vec4<T>& q, T kv, T av[3]) {
     const T c = harmonic(me.w, q.w) * kv;
