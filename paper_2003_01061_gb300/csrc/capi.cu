@@ -494,6 +494,9 @@ template <typename T> void set_cell_arrays(sph_batch* b) {
     s.occ = (unsigned*)take(b->occ_cap * 4 * OCCW);
     s.ncell = b->ncell;
     s.nocc = b->nocc;
+    s.levels = 1;
+    for (const Inst& I : b->in)
+        if (I.n > 0) s.levels = std::max(s.levels, I.grid.L);
 }
 
 template <typename T, int D> void repack(sph_batch* b) { launch_repack<T, D>(st<T>(b), b->d_old_off, b->d_move_n, b->stream); }

@@ -1,7 +1,7 @@
 // interact.cu -- the fused pressure pass of one relaxation step (Algorithm 1: renormalisation
 // gamma_i, pressure force with the feature-boundary correction, map onto the feature, step-size
 // candidates) over the neighbour lists of the search (search.cu).  LPP consecutive lanes handle
-// one particle (sorted order) and split its list, LISTU consecutive entries per lane and turn;
+// one particle (sorted order) and split its list, a few consecutive entries per lane and turn;
 // their partial sums are combined with a fixed shuffle butterfly.
 //
 // For particle i of group g (intrinsic dimension d, kernel W_d, rho = h^-d, P = p0 h^(2d)):
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(BLOCK, (interact_minb<T, D>()))
     k_interact(const __grid_constant__ State<T> s, const __grid_constant__ One one, T* dbg_sigma, T* dbg_gamma, int cls) {
     dep_launch();
     dep_wait();
-    constexpr int LPP = Lpp<D>::v, CL = 32 / LPP, U = LISTU;
+    constexpr int LPP = Lpp<D>::v, CL = 32 / LPP, U = pressure_listu<D>();
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ SearchWarp<CL> ww[BLOCK / 32];
     __shared__ Grid gsh;

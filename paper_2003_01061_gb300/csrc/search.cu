@@ -63,7 +63,7 @@ void launch_search_cl(const State<T>& s, const One* one, cudaStream_t st, bool p
 }
 template <typename T, int D>
 void launch_search(const State<T>& s, const One* one, cudaStream_t st, bool pdl, int cls, unsigned long long* tested) {
-    const int cl = search_width(D, s.n);
+    const int cl = search_width(D, s.n, s.levels);
     if constexpr (D == 3)
         if (cl == 2) return launch_search_cl<T, D, 2>(s, one, st, pdl, cls, tested);
     if (cl == 4) launch_search_cl<T, D, 4>(s, one, st, pdl, cls, tested);

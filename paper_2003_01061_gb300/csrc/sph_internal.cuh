@@ -19,6 +19,7 @@ constexpr int CHUNK = SPH_SLOT_CHUNK;   // slot alignment of instances (a multip
 template <typename T> struct State {
     int n;             // total slots of the batch
     int NI;            // instances
+    int levels;        // most grid levels of a loaded instance
     const int* inst_off;    // [NI+1]
     const int* inst_n;      // [NI]
     const int* chunk_inst;  // [n / CHUNK] instance of every chunk of slots
@@ -118,9 +119,12 @@ template <int D> struct Lpp {
 // needs more, or any list with blocks in a chunk that ran out of them, counts as overflowed (which
 // lists got blocks there depends on timing, whether the chunk ran out does not): the pair passes
 // search those particles' neighbours again.
+// In 2D a row is one 128-byte line, and every particle of a chunk can have a block (measured, rows of
+// 32 with 128 blocks against rows of 48 with 64, the same memory, us per step: constant spacing, 127k
+// particles 113.3 / 110.8, 300k 210.7 / 204.0; 120k disk 132.9 / 130.5, 1M disk 627 / 614).
 template <int D> struct ListShape;
 template <> struct ListShape<2> {
-    static constexpr int ROW = 48, XB = 32, NXB = 64;
+    static constexpr int ROW = 32, XB = 32, NXB = 128;
 };
 template <> struct ListShape<3> {
     static constexpr int ROW = 128, XB = 64, NXB = 128;
@@ -131,29 +135,39 @@ template <int D> constexpr int list_most() { return ListShape<D>::ROW + XMAX * L
 template <int D> constexpr int list_entries() {
     return ListShape<D>::ROW + ListShape<D>::XB * ListShape<D>::NXB / CHUNK;
 }
-// consecutive list entries per lane and turn of the pair passes: their loads are in flight together
-// (measured on the 1.2M cube: 4 against 2 viscous sum and update 339 us against 468)
+// consecutive list entries per lane and turn of the viscous sum and of the pressure pass: their loads
+// are in flight together (measured on the 1.2M cube: 4 against 2 viscous sum and update 339 us against
+// 468).  A 2D list fills one and a half turns of 16 entries: the pressure pass takes turns of 8 (us per
+// step, 2 against 4: constant spacing, 127k particles 104.5 / 108.4, 300k 188.5 / 196.5; 120k disk 127.9
+// / 131.6, 1M disk 602 / 618; the viscous sum gains nothing, 128.6 / 127.9 and 606 / 602 on the disks).
 constexpr int LISTU = 4;
+template <int D> constexpr int pressure_listu() { return D == 2 ? 2 : LISTU; }
 // particles searched by one warp: 2 (in 3D), 4, 8 or 16 by the slots of the batch.
 // A warp searching for more particles reads the cells around them once for all, one searching for
 // fewer is done sooner, which counts while the GPU is not full.  The lists do not depend on it.
 // Measured, search and pressure pass in us with 2 / 4 / 8 / 16: a 26k ball in three passes (whole
 // step) 376 / 437 / 640 / 826; a 20k disk 33 / 29 / 38 / 55; 120k disk 106 / 76 / 66 / 79; 1M disk
 // - / - / 430 / 404; 83k cube 189 / 149 / 137 / 146; 300k cube 671 / 498 / 472 / -; 1.2M cube
-// 2447 / - / 1451 / 1408.
-constexpr int search_width(int D, int slots) {
-    return D == 3 && slots <= 32768 ? 2 : slots <= 65536 ? 4 : slots <= 524288 ? 8 : 16;
+// 2447 / - / 1451 / 1408.  In a 2D mesh of constant spacing (levels 1) all warps take alike, and the
+// wider ones pay earlier: 4 / 8 / 16, 40k particles 37.6 / 35.5 / -, 60k 46.3 / 41.9 / -, 127k 76 / 66 / 66,
+// 300k - / 127.5 / 124.0.
+constexpr int search_width(int D, int slots, int levels) {
+    return D == 3 && slots <= 32768 ? 2
+           : D == 2 && levels == 1 ? (slots <= 32768 ? 4 : slots <= 262144 ? 8 : 16)
+                                   : (slots <= 65536 ? 4 : slots <= 524288 ? 8 : 16);
 }
 // most slots of a batch whose prediction, viscous sum and update run as one kernel (FP32 build).
-// Measured, one kernel against three, us per step: the 2.6k square 48.6 against 52.2, a 20k disk
-// 77.2 against 79.8, a 120k disk 156.3 against 138.9; 3D, a 26k ball in three passes 372 against
-// 363.  In FP64 the neighbours' predictions cost more than the launches (2.9k square 116 against 110).
-// Six resident blocks per SM asked of the compiler: 20k disk 73.4 against 75.3 with four, 73.8 eight.
+// Measured, one kernel against three, us per step: the 2.6k square 48.6 against 52.2; constant spacing,
+// 38k particles 57.1 against 63.1, 55k 73.5 / 74.6, 64k 76.0 / 76.2, 90k 89.8 / 88.3, 127k 109 / 103; a 38k
+// disk 77.4 / 82.6, 55k 94.7 / 95.0, 65k 99.9 / 101.4, 90k 116.8 / 114.6; 3D, a 26k ball in three passes
+// 372 / 363.  In FP64 the neighbours' predictions cost more than the launches (2.9k square 116 / 110).
+// Eight resident blocks per SM asked of the compiler take 38,912 particles at once, six 29,184: 57.4
+// against 61.2 at 30k, 51.8 against 50.8 at 20k.
 #ifndef SPH_FUSED_MINB
-#define SPH_FUSED_MINB 6
+#define SPH_FUSED_MINB 8
 #endif
 #ifndef SPH_FUSED_MOST_2D
-#define SPH_FUSED_MOST_2D 32768
+#define SPH_FUSED_MOST_2D 65536
 #endif
 #ifndef SPH_FUSED_MOST_3D
 #define SPH_FUSED_MOST_3D 8192
