@@ -507,23 +507,27 @@ template <typename T> struct StepOf {
     }
 };
 
-// (v~, eta) of a moving particle of dimension di from its (a_p, V~) and (v, h) records
+// (v~, eta) of a moving particle of dimension di from its (a_p, V~) and (v, h) records.  Rounded
+// op by op, as the pair terms below: the one-kernel update predicts where it needs the values, the
+// other reads them from memory, which of them runs depends on the slots of the whole batch, and an
+// instance's result must not.
 template <typename T>
 __device__ __forceinline__ Vec4<T> predicted(const Params& p, const StepOf<T>& st, const Vec4<T>& a, const Vec4<T>& vh, int di) {
     const T v[3] = {vh.x, vh.y, vh.z}, ap[3] = {a.x, a.y, a.z};
     T vt[3];
     for (int c = 0; c < 3; ++c) {
-        const T vp = st.rs ? T(0) : st.f * v[c];
-        vt[c] = vp + st.dt * (ap[c] - st.eps * vp);
+        const T vp = st.rs ? T(0) : rn_mul(st.f, v[c]);
+        vt[c] = rn_fma(st.dt, rn_fma(-st.eps, vp, ap[c]), vp);
     }
     T hd, h2d;
     hpow(vh.w, di, hd, h2d);
+    const T nu = rn_mul(rn_mul(wp<T>(p.visc, p.visc_f), wp<T>(p.kappa, p.kappa_f)), vh.w);
+    const T speed = t_sqrt(rn_fma(vt[2], vt[2], rn_fma(vt[1], vt[1], rn_mul(vt[0], vt[0]))));
     Vec4<T> q;
     q.x = vt[0];
     q.y = vt[1];
     q.z = vt[2];
-    q.w = wp<T>(p.visc, p.visc_f) * wp<T>(p.kappa, p.kappa_f) * vh.w *
-          t_sqrt(vt[0] * vt[0] + vt[1] * vt[1] + vt[2] * vt[2]) * fast_rcp(hd);
+    q.w = rn_mul(rn_mul(nu, speed), fast_rcp(hd));
     return q;
 }
 
@@ -544,10 +548,10 @@ __global__ void __launch_bounds__(BLOCK) k_predict(State<T> s, One one, const Ct
 
 // the viscous term of Eq. 7 of a pair: me, q the two particles' (v~, eta), kv the kernel factor
 template <typename T, int D> __device__ __forceinline__ void visc_pair(const Vec4<T>& me, const Vec4<T>& q, T kv, T av[3]) {
-    const T c = harmonic(me.w, q.w) * kv;
-    av[0] += c * (me.x - q.x);
-    av[1] += c * (me.y - q.y);
-    if (D == 3) av[2] += c * (me.z - q.z);
+    const T c = rn_mul(harmonic(me.w, q.w), kv);
+    av[0] = rn_fma(c, rn_sub(me.x, q.x), av[0]);
+    av[1] = rn_fma(c, rn_sub(me.y, q.y), av[1]);
+    if (D == 3) av[2] = rn_fma(c, rn_sub(me.z, q.z), av[2]);
 }
 
 // the viscous sums of the warp's particles whose list overflowed (over), from a second search; all

@@ -136,6 +136,9 @@ __device__ __forceinline__ double rn_add(double a, double b) { return __dadd_rn(
 __device__ __forceinline__ double rn_sub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double rn_mul(double a, double b) { return __dmul_rn(a, b); }
 
+__device__ __forceinline__ float rn_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double rn_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 __device__ __forceinline__ unsigned long long min_bits(float v) { return (unsigned long long)__float_as_uint(v); }
 __device__ __forceinline__ unsigned long long min_bits(double v) { return (unsigned long long)__double_as_longlong(v); }
 template <typename T> __device__ __forceinline__ T from_bits(unsigned long long b);
@@ -495,8 +498,8 @@ template <typename T> __device__ __forceinline__ T kernel_factor(int d, T S2, T 
 
 // 2 a b / (a + b) for a, b >= 0 (0 where the sum is 0)
 template <typename T> __device__ __forceinline__ T harmonic(T a, T b) {
-    const T s = a + b;
-    return s > T(0) ? T(2) * a * b / s : T(0);
+    const T s = rn_add(a, b);
+    return s > T(0) ? rn_mul(rn_mul(T(2), a), b) / s : T(0);
 }
 
 // sum over the LPP lanes of one particle (xor butterfly: every lane gets the same bits).  The
