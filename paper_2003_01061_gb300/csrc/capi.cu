@@ -495,8 +495,12 @@ template <typename T> void set_cell_arrays(sph_batch* b) {
     s.ncell = b->ncell;
     s.nocc = b->nocc;
     s.levels = 1;
+    s.wide = false;
     for (const Inst& I : b->in)
-        if (I.n > 0) s.levels = std::max(s.levels, I.grid.L);
+        if (I.n > 0) {
+            s.levels = std::max(s.levels, I.grid.L);
+            s.wide = s.wide || I.grid.dims[0][0] > SEARCH_WRAP;
+        }
 }
 
 template <typename T, int D> void repack(sph_batch* b) { launch_repack<T, D>(st<T>(b), b->d_old_off, b->d_move_n, b->stream); }

@@ -324,7 +324,7 @@ template <typename T, int D, bool ONE> __global__ void __launch_bounds__(BLOCK) 
     const Params& p = ONE ? one.p : s.params[inst];
     const float ic0 = 1.0f / g.c0;
     float4 f;
-    f.x = fmaf((float)off[0], ic0, (float)corner[0]);
+    f.x = fmaf((float)off[0], ic0, (float)(corner[0] & (SEARCH_WRAP - 1)));
     f.y = fmaf((float)off[1], ic0, (float)corner[1]);
     f.z = D == 3 ? fmaf((float)off[2], ic0, (float)corner[2]) : 0.0f;
     f.w = (0.5f * p.kappa_f * ic0 * (1.0f + 0x1p-12f)) * (float)h;

@@ -9,7 +9,7 @@ namespace sph {
 // cls: the dimension class of the pass (in_pass), or -1 for every particle, whatever its dimension
 // or its instance's phase (inspection).  tested: if not null, the candidate pairs tested are
 // counted in it.
-template <typename T, int D, bool ONE, int CL>
+template <typename T, int D, bool ONE, int CL, bool WIDE>
 __global__ void __launch_bounds__(32 * search_warps(CL), 32 / search_warps(CL))
 k_search(State<T> s, One one, int cls, unsigned long long* tested) {
     dep_launch();
@@ -46,7 +46,7 @@ k_search(State<T> s, One one, int cls, unsigned long long* tested) {
         }
     }
     unsigned long long count = 0;
-    const int n = warp_search<T, D, CL, false>(g, s, ww, lane, k0, active, fi, li, ci, count, [](int) {});
+    const int n = warp_search<T, D, CL, false, WIDE>(g, s, ww, lane, k0, active, fi, li, ci, count, [](int) {});
     __syncwarp();
     if (sub == 0 && k < s.n) {
         s.vcnt[k] = n;
@@ -55,11 +55,16 @@ k_search(State<T> s, One one, int cls, unsigned long long* tested) {
     if (tested && lane == 0) atomicAdd(tested, count);
 }
 
+template <typename T, int D, int CL, bool WIDE>
+void launch_search_wide(const State<T>& s, const One* one, cudaStream_t st, bool pdl, int cls, unsigned long long* tested) {
+    const int nb = div_up(s.n, CL * search_warps(CL)), nt = 32 * search_warps(CL);
+    if (one) launch_k(k_search<T, D, true, CL, WIDE>, nb, nt, st, pdl, s, *one, cls, tested);
+    else launch_k(k_search<T, D, false, CL, WIDE>, nb, nt, st, pdl, s, One(), cls, tested);
+}
 template <typename T, int D, int CL>
 void launch_search_cl(const State<T>& s, const One* one, cudaStream_t st, bool pdl, int cls, unsigned long long* tested) {
-    const int nb = div_up(s.n, CL * search_warps(CL)), nt = 32 * search_warps(CL);
-    if (one) launch_k(k_search<T, D, true, CL>, nb, nt, st, pdl, s, *one, cls, tested);
-    else launch_k(k_search<T, D, false, CL>, nb, nt, st, pdl, s, One(), cls, tested);
+    if (s.wide) launch_search_wide<T, D, CL, true>(s, one, st, pdl, cls, tested);
+    else launch_search_wide<T, D, CL, false>(s, one, st, pdl, cls, tested);
 }
 template <typename T, int D>
 void launch_search(const State<T>& s, const One* one, cudaStream_t st, bool pdl, int cls, unsigned long long* tested) {

@@ -16,10 +16,17 @@ namespace sph {
 
 constexpr int CHUNK = SPH_SLOT_CHUNK;   // slot alignment of instances (a multiple of every pair-pass block)
 
+// Search records hold x modulo this many finest cells (y and z have fewer): beyond it single precision
+// would be too coarse, and the search radius, widened by its rounding, would take in whole cells of
+// strangers (2D ribbons of 2^18, 2^20 and 2^21 cells: 1,043, 4,064 and 8,074 us per step, with x as it is
+// 1,219, 10,424 and 32,887).  A search spans less than a quarter of it.
+constexpr int SEARCH_WRAP = 1 << 14;
+
 template <typename T> struct State {
     int n;             // total slots of the batch
     int NI;            // instances
     int levels;        // most grid levels of a loaded instance
+    bool wide;         // one of them has a grid longer than SEARCH_WRAP cells along x
     const int* inst_off;    // [NI+1]
     const int* inst_n;      // [NI]
     const int* chunk_inst;  // [n / CHUNK] instance of every chunk of slots
@@ -44,7 +51,8 @@ template <typename T> struct State {
     int* IDs;
     int* Ks;
     Vec4<T>* P;
-    float4* F;         // search records: position and kappa h / 2 in finest cells (padding: stale)
+    float4* F;         // search records: position (x modulo SEARCH_WRAP) and kappa h / 2 in finest
+                       // cells (padding: stale)
     Vec4<T>* A;
     // rebuild scratch: per-cell counts (down to zero after the scatter), cell starts, scan block
     // sums, and the sorted-slot -> stored-index permutation

@@ -205,10 +205,11 @@ __device__ __forceinline__ void stg_if_less(float a, float b, char* p, int j) {
 //
 // FLUSH = false: a list takes the first list_most hits, blocks beyond its row taken as they are
 // needed; returns the number of hits of the lane's particle, and adds the candidate pairs tested to
-// `tested`.  FLUSH = true (lists that
-// overflowed): whenever a row is nearly full, and at the end, work(n) is called by all lanes, with
-// n hits of the lane's particle in its row, and the rows start again.
-template <typename T, int D, int CL, bool FLUSH, typename F>
+// `tested`.  FLUSH = true (lists that overflowed): whenever a row is nearly full, and at the end,
+// work(n) is called by all lanes, with n hits of the lane's particle in its row, and the rows start
+// again.  WIDE = false: for grids of at most SEARCH_WRAP cells along x (the general form there: a step
+// of the 300k cube 599 us against 590).
+template <typename T, int D, int CL, bool FLUSH, bool WIDE = true, typename F>
 __device__ __forceinline__ int warp_search(const Grid& g, const State<T>& s, SearchWarp<CL>& ww, int lane, int k0,
                                            bool active, float4 fi, int li, const int ci[3],
                                            unsigned long long& tested, F&& work) {
@@ -221,10 +222,10 @@ __device__ __forceinline__ int warp_search(const Grid& g, const State<T>& s, Sea
     constexpr unsigned NEAR_F = sizeof(float4) * CL, NEAR_J = NEAR_F + 64 * sizeof(float4), DELTA = NEAR_J + 256;
     char* const list = reinterpret_cast<char*>(s.vj + (size_t)k0 * ROW);
     // Search records are off by less than 2^-24 of the grid's extent X per coordinate and
-    // particle, their difference and the exact predicate's own rounding by as much again: less
-    // than 2^-20.6 X in the distance.  A pair's radius is widened by 2^-20 X here, and by a
-    // relative 2^-12 where the record is written.
-    const float pad = (float)max(g.dims[0][0], max(g.dims[0][1], g.dims[0][2])) * 0x1p-20f;
+    // particle (X at most SEARCH_WRAP cells), their difference and the exact predicate's own rounding
+    // by as much again: less than 2^-20.6 X in the distance.  A pair's radius is widened by 2^-20 X
+    // here, and by a relative 2^-12 where the record is written.
+    const float pad = (float)max(min(g.dims[0][0], SEARCH_WRAP), max(g.dims[0][1], g.dims[0][2])) * 0x1p-20f;
     unsigned end[CL];   // byte offset in `list` of the next hit of every particle
 #pragma unroll
     for (int q = 0; q < CL; ++q) end[q] = q * ROW * 4;
@@ -267,7 +268,18 @@ __device__ __forceinline__ int warp_search(const Grid& g, const State<T>& s, Sea
                         (D == 2 || ci[2] == sc[2]) && (unsigned)(ci[0] - sc[0]) <= (unsigned)seg_span(D, CL);
         const unsigned seg = __ballot_sync(FULL, in && sub == 0);
         pend &= ~seg;
-        const float x[3] = {fi.x, fi.y, fi.z};
+        // x counts from x0, in grids beyond SEARCH_WRAP a quarter of it before the segment, where the
+        // records' x start again in between
+        const bool wide = WIDE && g.dims[0][0] > SEARCH_WRAP;
+        const int x0 = wide ? (sc[0] << sl) - SEARCH_WRAP / 4 : 0;
+        auto from_x0 = [&](float v) {
+            if (wide) {
+                v -= (float)(x0 & (SEARCH_WRAP - 1));
+                v = v < 0.0f ? v + (float)SEARCH_WRAP : v;
+            }
+            return v;
+        };
+        const float x[3] = {from_x0(fi.x), fi.y, fi.z};
         float b0[3] = {0, 0, 0}, b1[3] = {0, 0, 0};
         for (int a = 0; a < D; ++a) {
             b0[a] = warp_min_nn(in ? fmaxf(x[a], 0.0f) : 3e38f);
@@ -295,8 +307,9 @@ __device__ __forceinline__ int warp_search(const Grid& g, const State<T>& s, Sea
                 auto box = [&]() -> bool {
                     bool some = true;
                     for (int a = 0; a < D; ++a) {
-                        lo[a] = max(__float2int_rd(b0[a] - R) >> l, 0);
-                        hb[a] = min(__float2int_rd(b1[a] + R) >> l, g.dims[l][a] - 1);
+                        const int s0 = a == 0 ? x0 : 0;
+                        lo[a] = max((__float2int_rd(b0[a] - R) + s0) >> l, 0);
+                        hb[a] = min((__float2int_rd(b1[a] + R) + s0) >> l, g.dims[l][a] - 1);
                         some = some && lo[a] <= hb[a];
                     }
                     return some;
@@ -386,8 +399,8 @@ __device__ __forceinline__ int warp_search(const Grid& g, const State<T>& s, Sea
                 const float rem = fmaf(Rl, Rl, -d2);
                 if (rem > 0.0f) {
                     const float w = rem * rsqrtf(rem);
-                    const int a0 = max(__float2int_rd(b0[0] - w) >> l, lol[0]);
-                    const int a1 = min(__float2int_rd(b1[0] + w) >> l, hxl);
+                    const int a0 = max((__float2int_rd(b0[0] - w) + x0) >> l, lol[0]);
+                    const int a1 = min((__float2int_rd(b1[0] + w) + x0) >> l, hxl);
                     if (a0 <= a1) {
                         const int row = g.base[l] + (cz * g.dims[l][1] + cy) * g.dims[l][0];
                         first = max(__ldg(s.cell_start + row + a0), 0);
@@ -418,7 +431,8 @@ __device__ __forceinline__ int warp_search(const Grid& g, const State<T>& s, Sea
                     started += __popc(heads);
                     // past the end: the last candidate again
                     const int j = min(c + lane, total - 1) + lds_i(sh_me + DELTA + 4 * ord);
-                    const float4 f = s.F[j];
+                    float4 f = s.F[j];
+                    f.x = from_x0(f.x);
                     const bool there = c + lane < total;
                     c += 32;
                     const float dx = fmaxf(fmaxf(b0[0] - f.x, f.x - b1[0]), 0.0f);
