@@ -146,7 +146,7 @@ struct sph_batch {
     void* cpool = nullptr;            // per-cell arrays
     void* stage = nullptr;            // the caller's arrays on the device (set_state, positions)
     size_t stage_cap = 0;
-    char* pin = nullptr;              // PIN_BYTES of pinned memory for reading small states back
+    std::vector<char> small;          // a small state read back (ONE_COPY_BYTES, from the first on)
     State<float> sf;
     State<double> sd;
     Grid* d_grids = nullptr;
@@ -637,7 +637,6 @@ void batch_free(sph_batch* b) {
     cudaFree(b->pool);
     cudaFree(b->cpool);
     cudaFree(b->stage);
-    cudaFreeHost(b->pin);
     cudaFree(b->d_grids);
     cudaFree(b->d_params);
     cudaFree(b->d_doms);
@@ -850,11 +849,12 @@ char* stage_buf(sph_batch* b, size_t bytes) {
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// States of up to this many staged bytes are read back in one copy through pinned memory instead of
-// one copy per array to pageable memory, whose call overhead is what such a read costs (measured,
-// positions() of 2.6k particles, 156 KB, 41 us against 66; of 20k, 1.2 MB, 107 against 90: there
-// the copies count, and the driver's straight way to the caller's pages is the faster one)
-constexpr size_t PIN_BYTES = 256 * 1024;
+// States of up to this many staged bytes are read back in one copy instead of one per array, whose
+// call overhead is what such a read costs (measured, positions() of 2.6k particles, 156 KB, 41 us
+// against 69, the first of a handle 56 against 82; through pinned memory 46, but 165 for the first and
+// 150 more to free it; of 20k, 1.2 MB, 107 against 90: there the copies count, and the driver's
+// straight way to the caller's pages is the faster one)
+constexpr size_t ONE_COPY_BYTES = 256 * 1024;
 
 IoGrid io_grid(const Inst& I) {
     IoGrid g;
@@ -901,18 +901,16 @@ sph_status download(sph_batch* b, int inst, int* const Cd[3], T* const Od[3], T*
     CK(cudaGetLastError());
     int hc[2] = {0, 0};
     const size_t staged = 256 + 2 * nx + nh + (size_t)n * 4;
-    if (staged <= PIN_BYTES && !b->pin && cudaHostAlloc(&b->pin, PIN_BYTES, cudaHostAllocDefault) != cudaSuccess) {
-        cudaGetLastError();
-        b->pin = nullptr;
-    }
-    if (staged <= PIN_BYTES && b->pin) {
-        CK(cudaMemcpyAsync(b->pin, p, staged, cudaMemcpyDeviceToHost, b->stream));
+    if (staged <= ONE_COPY_BYTES) {
+        b->small.resize(ONE_COPY_BYTES);
+        const char* const q = b->small.data();
+        CK(cudaMemcpyAsync(b->small.data(), p, staged, cudaMemcpyDeviceToHost, b->stream));
         CK(cudaStreamSynchronize(b->stream));
-        std::memcpy(hc, b->pin, 8);
-        if (x_out) std::memcpy(x_out, b->pin + 256, (size_t)n * 24);
-        if (v_out) std::memcpy(v_out, b->pin + 256 + nx, (size_t)n * 24);
-        if (h_out) std::memcpy(h_out, b->pin + 256 + 2 * nx, (size_t)n * 8);
-        if (group_out) std::memcpy(group_out, b->pin + 256 + 2 * nx + nh, (size_t)n * 4);
+        std::memcpy(hc, q, 8);
+        if (x_out) std::memcpy(x_out, q + 256, (size_t)n * 24);
+        if (v_out) std::memcpy(v_out, q + 256 + nx, (size_t)n * 24);
+        if (h_out) std::memcpy(h_out, q + 256 + 2 * nx, (size_t)n * 8);
+        if (group_out) std::memcpy(group_out, q + 256 + 2 * nx + nh, (size_t)n * 4);
         if (hc[1] != 0 || hc[0] != n) return fail(SPH_E_CUDA, "corrupt particle index on the device");
         return SPH_OK;
     }
