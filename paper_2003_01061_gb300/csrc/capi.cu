@@ -487,7 +487,6 @@ template <typename T> void set_cell_arrays(sph_batch* b) {
     };
     s.count = (int*)take(b->cell_cap * 4);
     s.cell_start = (int*)take((b->cell_cap + 1) * 4);
-    s.bsum = (int*)take((size_t)SCAN_TILE * 4);
     s.tstate = (unsigned long long*)take((size_t)div_up((long long)b->cell_cap, SCAN1_TILE) * 8);
     s.ticket = (int*)take(4);
     s.ntile = div_up(b->ncell, SCAN1_TILE);
@@ -543,8 +542,8 @@ sph_status relayout(sph_batch* b, int changed, int new_n, int desc) {
     if (!b->cpool || (size_t)keys > b->cell_cap || (size_t)occ > b->occ_cap) {
         const size_t kc = std::max({(size_t)keys, b->cell_cap, (size_t)1});
         const size_t oc = std::max({(size_t)occ, b->occ_cap, (size_t)1});
-        const size_t bytes = kc * 4 + (kc + 1) * 4 + (size_t)SCAN_TILE * 4 + oc * 4 * OCCW +
-                             (size_t)div_up((long long)kc, SCAN1_TILE) * 8 + 4 + 6 * 256;
+        const size_t bytes = kc * 4 + (kc + 1) * 4 + oc * 4 * OCCW +
+                             (size_t)div_up((long long)kc, SCAN1_TILE) * 8 + 4 + 5 * 256;
         void* p = nullptr;
         if (cudaMalloc(&p, bytes) != cudaSuccess)
             return fail(SPH_E_NOMEM, "device allocation of %zu bytes of cell arrays failed", bytes);

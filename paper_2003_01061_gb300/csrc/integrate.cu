@@ -10,16 +10,6 @@ __device__ __forceinline__ double rel_err(double a, double b) {
     return a == 0.0 ? 0.0 : CUDART_INF;
 }
 
-__device__ inline void window_reset(Ctrl* c) {
-    c->wcount = 0;
-    c->nwin = 0;
-    for (int g = 0; g < MAXF; ++g) {
-        c->wsum[g] = 0.0;
-        c->A_last[g] = 0.0;
-        c->A_prev[g] = 0.0;
-    }
-}
-
 constexpr int CTL_THREADS = 512;   // threads of the controller's block
 constexpr int CTL_GP = 8;          // groups summed per pass of the sampling reduction
 

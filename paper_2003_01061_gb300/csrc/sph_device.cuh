@@ -161,13 +161,6 @@ template <typename T> __device__ __forceinline__ T wp(double d, float f);
 template <> __device__ __forceinline__ float wp<float>(double, float f) { return f; }
 template <> __device__ __forceinline__ double wp<double>(double d, float) { return d; }
 
-// h^k for small non-negative integer k
-template <typename T> __device__ __forceinline__ T ipow(T h, int k) {
-    T r = T(1);
-    for (int i = 0; i < k; ++i) r *= h;
-    return r;
-}
-
 // h^d and h^(2d) for an intrinsic dimension d in {1, 2, 3}
 template <typename T> __device__ __forceinline__ void hpow(T h, int d, T& hd, T& h2d) {
     const T h2 = h * h;
@@ -306,17 +299,6 @@ __device__ __forceinline__ void level_repr(const Grid& g, int l, const int c[3],
 
 __device__ __forceinline__ int key_of(const Grid& g, int l, const int cell[3]) {
     return g.base[l] + (cell[2] * g.dims[l][1] + cell[1]) * g.dims[l][0] + cell[0];
-}
-
-// decode a key into level and cell coordinates
-__device__ __forceinline__ void decode_key(const Grid& g, int key, int& l, int cell[3]) {
-    l = 0;
-    while (l < g.L - 1 && key >= g.base[l + 1]) ++l;
-    int r = key - g.base[l];
-    cell[0] = r % g.dims[l][0];
-    r /= g.dims[l][0];
-    cell[1] = r % g.dims[l][1];
-    cell[2] = r / g.dims[l][1];
 }
 
 // ---- analytic geometry (FP64) ----

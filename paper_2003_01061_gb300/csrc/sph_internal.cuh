@@ -54,11 +54,9 @@ template <typename T> struct State {
     float4* F;         // search records: position (x modulo SEARCH_WRAP) and kappa h / 2 in finest
                        // cells (padding: stale)
     Vec4<T>* A;
-    // rebuild scratch: per-cell counts (down to zero after the scatter), cell starts, scan block
-    // sums, and the sorted-slot -> stored-index permutation
+    // rebuild scratch: per-cell counts (down to zero after the scatter) and cell starts
     int* count;
     int* cell_start;
-    int* bsum;
     // one-pass scan: per-tile status words (flag << 62 | value) and the tile ticket, cleared by
     // whichever kernel produces the histogram
     unsigned long long* tstate;
