@@ -226,31 +226,43 @@ __device__ __forceinline__ bool inside(const Domain& dm, const double x[3], cons
     return samp_phi(dm, x) > 0.0;
 }
 
-// h_t(x) of a point of the volume, bit for bit as samp_h has it: with several reference circles or
-// spheres, only the nearest one's distance is formed in FP64 where single precision shows which it
-// is (by far more than its rounding, 2^-20 of the domain's size).
-__device__ __forceinline__ double quad_h(const Sizing& z, const double x[3], const float xf[3], float size) {
-    if (z.kind != 1 || z.nref < 2) return samp_h(z, x);
-    float best = 3e38f, next = 3e38f;
-    int kb = 0;
-    for (int k = 0; k < z.nref; ++k) {
-        float s = 0.0f;
-        for (int a = 0; a < 3; ++a) s = fmaf(xf[a] - z.frc[k][a], xf[a] - z.frc[k][a], s);
-        const float d = fabsf(sqrtf(s) - z.frr[k]);
-        if (d < best) {
-            next = best;
-            best = d;
-            kb = k;
-        } else {
-            next = fminf(next, d);
+// h_t(x) of a point of the volume, bit for bit as samp_h has it (sx2: (x_0 - c_0)^2 of the one
+// reference, formed before the loop).  With several reference circles or spheres, only the nearest
+// one's distance is formed in FP64 where single precision shows which it is (by far more than its
+// rounding, 2^-20 of the domain's size).
+__device__ __forceinline__ double quad_h(const Sizing& z, const double x[3], const float xf[3], float size, double sx2) {
+    if (z.kind != 1 || z.nref < 1) return samp_h(z, x);
+    double d;
+    if (z.nref == 1) {
+        const double d1 = dsub(x[1], z.rc[0][1]), d2 = dsub(x[2], z.rc[0][2]);
+        d = fabs(dsub(__dsqrt_rn(dadd(dadd(sx2, dmul(d1, d1)), dmul(d2, d2))), z.rr[0]));
+    } else {
+        float best = 3e38f, next = 3e38f;
+        int kb = 0;
+        for (int k = 0; k < z.nref; ++k) {
+            float s = 0.0f;
+            for (int a = 0; a < 3; ++a) s = fmaf(xf[a] - z.frc[k][a], xf[a] - z.frc[k][a], s);
+            const float dk = fabsf(sqrtf(s) - z.frr[k]);
+            if (dk < best) {
+                next = best;
+                best = dk;
+                kb = k;
+            } else {
+                next = fminf(next, dk);
+            }
         }
+        if (!(next - best > size * 0x1p-16f)) return samp_h(z, x);
+        d = fabs(dsub(dist_n(x, z.rc[kb], 3), z.rr[kb]));
     }
-    if (!(next - best > size * 0x1p-16f)) return samp_h(z, x);
-    double h = dadd(z.a, dmul(z.b, fabs(dsub(dist_n(x, z.rc[kb], 3), z.rr[kb]))));
+    double h = dadd(z.a, dmul(z.b, d));
     if (h < z.lo) h = z.lo;
     if (h > z.hi) h = z.hi;
     return h;
 }
+
+// i + 1/2 for 0 <= i < 2^31, exactly, in one FP64 subtraction (a conversion from an integer runs on the
+// same narrow pipe, and the addition comes on top)
+__device__ __forceinline__ double mid(int i) { return dsub(__hiloint2double(0x43300000, i), 4503599627370495.5); }
 
 // Midpoint-rule integral of rho_t over feature k (Eqs. 10, 11), per-block partial sums.  The
 // quadrature sizes are powers of two (nq = 2^ln), so the divisions by nq are exact and a point's
@@ -261,8 +273,11 @@ __device__ __forceinline__ double quad_h(const Sizing& z, const double x[3], con
 // whatever its size.  (Roots and reciprocals by one Newton step, within an ulp, and fewer blocks for
 // the small features gave other counts in 14 of 821 such features.)
 // Bound by the FP64 pipe, two multiply-adds per SM and clock: a volume point costs one root and one
-// quotient.  All features of a cube take 2.19 ms, of a disk 0.43 (one launch per feature, with
-// quotients per point for the cell size and a second root for the level set: 4.41 and 1.49).
+// quotient, and two coordinates, since a thread's points share their first one (its stride is a
+// multiple of nq); the single-precision coordinates that decide the filters come from the indices.
+// All features of a cube take 1.82 ms, of a disk 0.35 (coordinates and conversions per point: 2.19
+// and 0.43; one launch per feature, with quotients per point for the cell size and a second root for
+// the level set: 4.41 and 1.49).
 constexpr int QUAD_BLOCKS = 4 * 152;
 template <int KIND>
 __device__ __forceinline__ double integral_share(const Domain& dm, const Sizing& z, const Feat& f, long long npts, int ln,
@@ -293,17 +308,30 @@ __device__ __forceinline__ double integral_share(const Domain& dm, const Sizing&
     }
     if (KIND == SPH_FEAT_CIRCLE) cell = 2.0 * CUDART_PI * f.g[2] * inq;
     if (KIND == SPH_FEAT_RECT) cell = (f.g[9] * inq) * (f.g[10] * inq);
+    double x0 = 0.0, sx2 = 0.0;
+    float xf0 = 0.0f, dxf[3] = {0.0f, 0.0f, 0.0f};
+    if (KIND == SPH_FEAT_VOLUME) {
+        static_assert(QUAD_BLOCKS * SB % SPH_QUAD_VOLUME == 0 && QUAD_BLOCKS * SB % SPH_QUAD_AREA == 0,
+                      "the points of a thread share their first coordinate");
+        x0 = fma(mid((block * SB + (int)threadIdx.x) & last), dx[0], dm.lo[0]);
+        xf0 = (float)x0;
+        const double d0 = dsub(x0, z.rc[0][0]);
+        sx2 = dmul(d0, d0);
+        for (int a = 0; a < D; ++a) dxf[a] = (float)dx[a];
+    }
     double acc = 0.0;
     for (long long i = (long long)block * SB + threadIdx.x; i < npts; i += (long long)QUAD_BLOCKS * SB) {
         double x[3] = {0.0, 0.0, 0.0};
         if (KIND == SPH_FEAT_VOLUME) {
-            float xf[3];
-            for (int a = 0; a < 3; ++a) {
-                if (a < D) x[a] = dm.lo[a] + (((int)(i >> (a * ln)) & last) + 0.5) * dx[a];
-                xf[a] = (float)x[a];
+            x[0] = x0;
+            float xf[3] = {xf0, 0.0f, 0.0f};
+            for (int a = 1; a < D; ++a) {
+                const int ia = (int)(i >> (a * ln)) & last;
+                x[a] = fma(mid(ia), dx[a], dm.lo[a]);
+                xf[a] = fmaf((float)ia + 0.5f, dxf[a], dm.flo[a]);
             }
             if (inside(dm, x, xf, size)) {
-                const double h = quad_h(z, x, xf, size);
+                const double h = quad_h(z, x, xf, size, sx2);
                 acc += cell / (D == 3 ? h * h * h : h * h);
             }
         } else if (KIND == SPH_FEAT_SEGMENT) {
