@@ -63,7 +63,7 @@ FLOP_PER_PAIR = 50.0       # FP32 operations per interacting pair of the pressur
 # particles, 5 steps after the start; the traffic grows with the particle count (own state,
 # neighbour records missing L2, the neighbour lists), so a step on n particles moves n times this.
 # Set to None whenever the kernels change until they have been captured again.
-DOMINANT_DRAM_BYTES_PER_PARTICLE = (27.692288e6 + 54.203392e6 + 133.530624e6 + 75.097600e6) / 300_009
+DOMINANT_DRAM_BYTES_PER_PARTICLE = (27.747584e6 + 53.906432e6 + 133.533952e6 + 75.212032e6) / 300_009
 SM_COUNT, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 # one step of the headline: one-pass scan, scatter, gather, neighbour search, pressure pass,
 # controller, prediction, viscous sum, update (+ next keys)

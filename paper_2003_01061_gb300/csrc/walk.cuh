@@ -182,13 +182,13 @@ __device__ __forceinline__ void stg_if_less(float a, float b, char* p, int j) {
 // shared memory, two particles per packed operation).  The hits of a particle are appended, in
 // candidate order, to its row of the neighbour lists.
 //
-// What bounds it: the instruction stream, about 6k warp instructions per 8 particles on a 300k cube
-// (issue slots 73 % busy), a third of it in the ~27 groups of candidates, a third in the ~10 groups
+// What bounds it: the instruction stream, about 5.5k warp instructions per 8 particles on a 300k cube
+// (issue slots 68 % busy), a third of it in the ~27 groups of candidates, a third in the ~10 groups
 // tested, the rest in segments and rows; on small states the slowest warp's chain of loads.
 // Loading the next candidates ahead of the tests gained nothing at 32 warps per SM (605 us per step
 // with, 597 without, on that cube).  The walk it replaces, 8 lanes searching for
 // their own particle and working off its pairs as they came, took 2.9k per particle for search and
-// pair sums together (pressure pass of the 1.2M cube 3.6 ms; search and pressure pass now 1.47 ms).
+// pair sums together (pressure pass of the 1.2M cube 3.6 ms; search and pressure pass now 1.38 ms).
 // Measured on the way: testing every candidate against all particles without the box test 211 M
 // instead of 172 M instructions on that cube; pair sums inside the search kernel, from pools in
 // shared memory, 80 registers with spills in both and 1.8 ms.
